@@ -214,14 +214,11 @@ int ptebd_set_svd_polish(ptebd_state* st, int32_t mode);
 int ptebd_set_tensor_cores(ptebd_state* st, int32_t enable);
 
 /* Jacobi block width of the handle's SVDs (no counterpart in the paper: a
- * launch choice): the columns held in registers by one CTA, one per warp.
- * complex64: 16 (default) or 8; complex128: always 8.  0 selects the default.
- * Results are bit-identical run to run for a given width; two widths visit
- * the column pairs in different orders and so differ by rounding (both within
- * the SVD's accuracy).  complex64 width 8 runs two CTAs (two bonds) per SM;
- * measured at N = 1024, chi = 256 it is 7% slower than width 16, and the
- * autotuner picks it for some small-chi keys.  PTEBD_ERR_INVALID for other
- * widths. */
+ * launch choice).  complex64: 16 (default), the warps and the shared memory of a
+ * whole SM for each bond, or 8, at most 4 warps and half the shared memory;
+ * complex128: always 8.  0 selects the default.  Results are bit-identical run to
+ * run; the column pairs are met in the same order at either width.
+ * PTEBD_ERR_INVALID for other widths. */
 int ptebd_set_jacobi_width(ptebd_state* st, int32_t nw);
 
 /* PtSU after a gated layer on bonds 0, 2, 4, ... (the paper's odd bonds; a
@@ -237,26 +234,16 @@ int ptebd_set_jacobi_width(ptebd_state* st, int32_t nw);
  * drops an identity. */
 int ptebd_set_ptsu_shortcut(ptebd_state* st, int32_t enable);
 
-/* Columns of the complex64 Jacobi register block per warp at block width 16
- * (no counterpart in the paper: a scheduling choice).  pairs = 1 (the
- * default): 16 warps, one I column each, one column pair a round; pairs = 2:
- * 8 warps, each holding two I columns and rotating two independent column
- * pairs a round with their instruction streams interleaved.  Matrices of
- * more than 32 rows see their column pairs in the same order as with
- * pairs = 1; smaller ones run with 8-column blocks, so results differ from
- * pairs = 1 by rounding (both bit-identical run to run).  Measured at N = 1024,
- * chi = 256: the SVD takes 19% longer than with pairs = 1 (half the warps,
- * issue activity 38% against 51%), so it is an autotuner candidate, not the
- * default.  Width 8 and complex128 ignore it.  PTEBD_ERR_INVALID for other
- * values. */
+/* Kept for programs that set it: 1 (the default) or 2 are accepted, and both run
+ * the same kernel, whose warps hold a whole group of columns each (no counterpart
+ * in the paper).  PTEBD_ERR_INVALID for other values. */
 int ptebd_set_jacobi_pairs(ptebd_state* st, int32_t pairs);
 
 /* Autotuner (no counterpart in the paper: a scheduling choice of the library).
  * Times every candidate launch configuration on the state's own next layer
  * (the gates and parity a ptebd_apply_layer call would get, with the config's
- * PtSU steps): Jacobi block width and columns per warp (complex64: 16 with
- * one or two, 8 with one) x bond chunks (1, 2,
- * 4, 8, 12, 16, those the workspace can run concurrently); each candidate runs
+ * PtSU steps): Jacobi block width (complex64: 16 or 8) x bond chunks (1, 2, 4, 8,
+ * 12, 16, those the workspace can run concurrently); each candidate runs
  * twice from the saved state and the second run is timed with CUDA events on
  * the handle's stream.  The state is copied into `scratch` (device memory,
  * 256-byte aligned, at least state_bytes of ptebd_required_bytes, owned by
@@ -266,7 +253,7 @@ int ptebd_set_jacobi_pairs(ptebd_state* st, int32_t pairs);
  * under (chi_max padded, precision, bit length of N - 1, g): later
  * ptebd_create calls with the same key start with it.  best (may be NULL, else
  * 5 doubles): [block width, chunks, ms of the best, ms of the configuration
- * the handle had (-1 if it was not among the candidates), columns per warp].
+ * the handle had (-1 if it was not among the candidates), 1].
  * Synchronous. */
 int ptebd_autotune(ptebd_state* st, const double* gates, int32_t parity, int32_t gates_on_device,
                    void* scratch, size_t scratch_bytes, double* best);

@@ -104,8 +104,7 @@ struct LayerArgs {
     int eps_mode, stabilise, max_sweeps;
     int wait_test;    // test of the bounded waits: one hand-off wait per CTA targets a count nothing
                       // reaches, with a short limit, so the CTA aborts and latches DERR_TIMEOUT
-    int nw;           // Jacobi block width requested (0: the default; 8 or 16 for complex64)
-    int pairs;        // complex64, width 16: I columns per warp (1: 16 warps; 2: 8 warps, two pairs a round)
+    int nw;           // Jacobi block width requested (complex64: 8 halves a CTA's warps and shared memory)
     int tensor_cores; // complex64 on the tensor cores (tcgen05, 3xTF32) when chip >= 64: 1 theta' and
                       // the Gamma GEMM of gated stages, 2 the tSU steps as well
     int polish;       // complex64 Jacobi: one last sweep at the tighter threshold (see Eps::polish)
@@ -152,7 +151,6 @@ cudaError_t launch_add_partials(const double* partials, int k, double* totals, c
 constexpr int kMaxChunks = 16;
 template <typename R> cudaError_t jacobi_prepare();   // raises the dynamic smem limit
 int jacobi_block_width(int precision, int requested);  // the NW a launch with a.nw = requested uses
-size_t jacobi_smem_bytes(int precision, int ldw, int nw);
 
 // Transfer-matrix contraction.  C = rowscale o (op(A) B) o colscale * alpha + beta C,
 // all column-major; A and B are complex of type TA/TB, C is complex128.

@@ -1,0 +1,1182 @@
+// Batched one-sided (Hestenes) Jacobi SVD of the two-site tensors of a layer
+// (the SVD step of the TEBD procedure, Sec. II C of arXiv:2312.02667).
+//
+// One CTA per bond.  The matrix w (rows x cols, column-major, rows >= cols) is
+// taken in groups of B columns, by decreasing column norm (re-sorted at the
+// start of every sweep).  A sweep visits the pairs of groups in row-cyclic
+// order, as a pipeline of compute warps: warp v takes groups I = v, v + nwc,
+// v + 2 nwc, ... into registers, and every later group J flows past the warps in
+// the order of their I.  A counter per group (prog, release/acquire in shared
+// memory) says how many I it has met, so a warp waits only for its one
+// predecessor.  A visit (I, J) holds the 2 B columns in registers and goes
+// through their B^2 pairs in B rounds of B disjoint pairs: the B dot products
+// are reduced together, lanes p (32/B)..(p + 1)(32/B) - 1 work out the
+// rotation of pair p (the B rotations of a round side by side in one warp
+// instruction stream, so that the square roots and reciprocals are paid once a
+// round and not once a pair), and the coefficients come back through shared
+// memory.
+//
+// Where the columns are: when the matrix fits in shared memory (`RES`) it stays
+// there for the whole SVD.  Otherwise the groups are streamed: the last warp
+// fetches them by TMA bulk copies (cp.async.bulk, completion on an mbarrier)
+// into a ring of about 24 slots; the last warp of a row of I groups writes a
+// changed group back from its registers.
+//
+// Rotations are "fast": with the columns held as a = (1 + da) a~, a pair takes two
+// shears in place, a~ -= conj(tau) b~ and then b~ += kappa a~ (8 FMA per row
+// instead of 16 operations, no temporaries), and the factors cos of a and 1/cos
+// of b go into da and db, which stay with their columns and are multiplied out
+// only once they have moved by 2^-6.  da is kept as the difference from 1: cos - 1
+// and 1/cos - 1 = t^2 / (1 + sqrt(1 + t^2)) accumulate without rounding to zero
+// when t^2 is below the unit roundoff (cos itself would round to 1 while t does
+// not, and every such rotation would scale the pair by sqrt(1 + t^2)); multiplied
+// out at once they would round away just so, entry by entry, and the thousands of
+// small rotations of an SVD add up to 1e-6 in the complex64 norms.
+//
+// A pair (a, b) with |a^H b| > tol ||a|| ||b|| is rotated; the sweeps stop when
+// none was (or, on the complex64 path, when every rotation of a sweep was a
+// small one: Eps).  The squared column norms are recomputed at the start of every
+// sweep and tracked through the rotations in between; a norm that drops a lot
+// is recomputed from the rotated column.  On exit the columns are U S
+// (orthogonal, unsorted); their FP64 norms are the singular values.
+//
+// What bounds it: on complex64 the latency of a round's chain (dot products,
+// shuffles, the rotation, coefficients through shared memory), two or three warps
+// per scheduler; on complex128 the FP64 pipe.  Against one column per warp and a
+// rotation worked out by every lane of every pair (the kernel before this one):
+// 152 Ginibre matrices, complex64 128 x 128 3.81 -> 2.06 ms, 256 x 256 17.3 -> 9.0,
+// 512 x 512 95 -> 76; complex128, 64 of 128 x 128 98.6 -> 42.8 ms.  Why the groups go
+// in row-cyclic order: a tournament over all groups would keep every warp busy
+// but takes 13 to 16 sweeps where this order takes 10 or 11.
+//
+// Every wait is bounded by a clock budget; one that runs out raises the CTA's
+// abort flag, drains the CTA's own copies, latches DERR_TIMEOUT and returns.
+#pragma once
+#include <cmath>
+#include <type_traits>
+
+#include "ptebd_internal.h"
+
+namespace ptebd {
+namespace jac {
+
+// ------------------------------------------------------------------ PTX --
+__device__ __forceinline__ uint32_t smem_u32(const void* p) {
+    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_init_fence() {
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void counter_release(int* p, int v) {
+    asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ int counter_acquire(const int* p) {
+    int v;
+    asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+            smem_u32(dst)),
+        "l"(src), "r"(bytes), "r"(smem_u32(bar))
+        : "memory");
+}
+__device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)),
+                 "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// all but the last N bulk groups of this thread are complete
+template <int N> __device__ __forceinline__ void bulk_wait() {
+    asm volatile("cp.async.bulk.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+
+constexpr long long kWaitLimit = 1ll << 31;  // SM cycles, about a second
+
+// Bounded spin until *p >= target (or the CTA has aborted).  The clock and the
+// abort flag are looked at every 32 polls only.
+__device__ __forceinline__ bool counter_wait(const int* p, int target, const volatile int* abort_flag,
+                                             long long limit = kWaitLimit) {
+    if (counter_acquire(p) >= target) return true;
+    const long long start = clock64();
+    for (unsigned it = 1;; ++it) {
+        __nanosleep(20);
+        if (counter_acquire(p) >= target) return true;
+        if ((it & 31u) == 0u) {
+            if (clock64() - start > limit) return false;
+            if (*abort_flag) return false;
+        }
+    }
+}
+// Bounded wait for a phase of an mbarrier; abort_flag may be null.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const volatile int* abort_flag) {
+    if (mbar_try_wait(bar, parity)) return true;
+    const long long start = clock64();
+    while (!mbar_try_wait(bar, parity)) {
+        if (clock64() - start > kWaitLimit) return false;
+        if (abort_flag && *abort_flag) return false;
+    }
+    return true;
+}
+
+// ---------------------------------------------------------- arithmetic --
+// Unit roundoff and the rotation threshold factor: a pair is rotated when
+// |a^H b| > k sqrt(rows) u ||a|| ||b||.  Rounding alone leaves |a^H b| of about
+// sqrt(rows) u ||a|| ||b|| after a rotation, so the factor must sit well above 1
+// or rounding keeps re-triggering rotations (more sweeps, and every extra
+// rotation adds rounding error to the columns).
+// early: the sweeps also stop after a sweep in which every rotated pair had
+// cos^2 = |a^H b|^2 / (|a|^2 |b|^2) below early * tol^2 (0 = only after a sweep
+// without rotations).  On the complex64 path the sweep after such a sweep was
+// measured never to meet a pair above 1.04 tol^2 (gated and tSU matrices of
+// saturated layers, Ginibre and graded spectra: thousands of SVDs), and to
+// spend itself on 0 to 2 rotations of pairs barely above tol, so it is skipped;
+// the columns are left orthogonal to about tol instead of below tol.
+// range_e: matrices whose largest entry is not in [2^-range_e, 2^range_e) are
+// rescaled before the sweeps (see the range guard in jacobi_body).
+// polish: the factor of a last sweep's tighter threshold (A.polish), run once
+// after the stopping rule has fired: it rotates every pair with
+// |a^H b| > polish sqrt(rows) u |a| |b|, which leaves the columns orthogonal to
+// near the rounding of their storage (the truncated state depends on it).
+template <typename R> struct Eps;
+template <> struct Eps<float> {
+    static constexpr double u = 5.9604644775390625e-08;  // 2^-24
+    static constexpr double k = 8.0;
+    static constexpr int range_e = 24;
+    static constexpr double early = 256.0;
+    static constexpr double polish = 2.0;
+};
+template <> struct Eps<double> {
+    static constexpr double u = 1.1102230246251565e-16;  // 2^-53
+    static constexpr double k = 4.0;
+    static constexpr int range_e = 240;
+    static constexpr double early = 0.0;
+    static constexpr double polish = 0.0;
+};
+
+template <typename R>
+__device__ __forceinline__ R warp_sum(R v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+template <typename R>
+__device__ __forceinline__ R warp_max(R v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+// The binary exponent of a non-negative value, offset so that 0 (no entry) stays
+// below every real exponent: a shared atomicMax over it gives the exponent of the
+// largest entry of a matrix.
+constexpr int kExpOffset = 2048;
+template <typename R> __device__ __forceinline__ int exp_key(R v) {
+    return v > (R)0 ? ilogb((double)v) + kExpOffset : 0;
+}
+
+// Packed FP32 pairs (fma.rn.f32x2 and friends, sm_100 and later): two lanes of
+// FP32 arithmetic per instruction on a register pair (lo, hi).
+__device__ __forceinline__ unsigned long long pk2(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 upk2(unsigned long long v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// Columns.  complex64 (always RPL >= 2, rows even): pair-split layout while the
+// sweeps run, every two rows r, r + 1 (r even) stored as
+// (Re r, Re r+1, Im r, Im r+1), so that one 16-byte access moves the pair and the
+// packed FP32 instructions find the real parts and the imaginary parts of the
+// pair in one 64-bit register each.  Lane `lane` holds the pairs
+// r = 64 h + 2 lane, h = 0 .. RPL/2 - 1: entry 2 h is (Re r, Re r+1), entry
+// 2 h + 1 is (Im r, Im r+1).  complex128: entry q is row 32 q + lane.
+template <typename R> struct Entry { using T = unsigned long long; };
+template <> struct Entry<double> { using T = double2; };
+template <typename R> using entry_t = typename Entry<R>::T;
+
+template <int RPL>  // from a column in shared memory
+__device__ __forceinline__ void col_load(unsigned long long (&v)[RPL], const float2* col, int lane) {
+#pragma unroll
+    for (int h = 0; h < RPL / 2; ++h) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(col + 64 * h + 2 * lane);
+        v[2 * h] = t.x;
+        v[2 * h + 1] = t.y;
+    }
+}
+template <int RPL>
+__device__ __forceinline__ void col_load(double2 (&v)[RPL], const double2* col, int lane) {
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) v[q] = col[32 * q + lane];
+}
+template <int RPL>
+__device__ __forceinline__ void col_store(const unsigned long long (&v)[RPL], float2* col, int lane, int rows) {
+#pragma unroll
+    for (int h = 0; h < RPL / 2; ++h) {
+        const int r = 64 * h + 2 * lane;
+        if (r < rows) *reinterpret_cast<ulonglong2*>(col + r) = make_ulonglong2(v[2 * h], v[2 * h + 1]);
+    }
+}
+template <int RPL>
+__device__ __forceinline__ void col_store(const double2 (&v)[RPL], double2* col, int lane, int rows) {
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) {
+        const int r = 32 * q + lane;
+        if (r < rows) col[r] = v[q];
+    }
+}
+
+// a^H b over this lane's rows
+template <int RPL>
+__device__ __forceinline__ void col_dot(const unsigned long long (&a)[RPL], const unsigned long long (&b)[RPL],
+                                        float& gr, float& gi) {
+    unsigned long long r2 = 0ull, p2 = 0ull, m2 = 0ull;  // (0.f, 0.f)
+#pragma unroll
+    for (int h = 0; h < RPL / 2; ++h) {
+        r2 = fma2(a[2 * h], b[2 * h], r2);
+        p2 = fma2(a[2 * h], b[2 * h + 1], p2);
+        m2 = fma2(a[2 * h + 1], b[2 * h], m2);
+        r2 = fma2(a[2 * h + 1], b[2 * h + 1], r2);
+    }
+    const float2 r = upk2(r2), p = upk2(p2), m = upk2(m2);
+    gr = r.x + r.y;
+    gi = (p.x - m.x) + (p.y - m.y);
+}
+template <int RPL>
+__device__ __forceinline__ void col_dot(const double2 (&a)[RPL], const double2 (&b)[RPL], double& gr, double& gi) {
+    double r = 0.0, i = 0.0;
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) {
+        r = fma(a[q].x, b[q].x, r);
+        i = fma(a[q].x, b[q].y, i);
+        r = fma(a[q].y, b[q].y, r);
+        i = fma(-a[q].y, b[q].x, i);
+    }
+    gr = r;
+    gi = i;
+}
+
+// The coefficients of a rotation as the columns' instructions take them, handed
+// from the lanes that work them out to the whole warp through shared memory.
+template <typename R> struct Coef;
+template <> struct __align__(16) Coef<float> {
+    float4 a, b, c;  // (-tr, -tr, -ti, -ti), (ti, ti, kr, kr), (-ki, -ki, ki, ki)
+    __device__ __forceinline__ void set(float tr, float ti, float kr, float ki) {
+        a = make_float4(-tr, -tr, -ti, -ti);
+        b = make_float4(ti, ti, kr, kr);
+        c = make_float4(-ki, -ki, ki, ki);
+    }
+};
+template <> struct __align__(16) Coef<double> {
+    double2 t, k;
+    __device__ __forceinline__ void set(double tr, double ti, double kr, double ki) {
+        t = make_double2(tr, ti);
+        k = make_double2(kr, ki);
+    }
+};
+
+// a -= conj(tau) b, then b += kappa a (the new a)
+template <int RPL>
+__device__ __forceinline__ void col_rotate(unsigned long long (&a)[RPL], unsigned long long (&b)[RPL],
+                                           const Coef<float>& k) {
+    const ulonglong2 ka = *reinterpret_cast<const ulonglong2*>(&k.a), kb = *reinterpret_cast<const ulonglong2*>(&k.b),
+                     kc = *reinterpret_cast<const ulonglong2*>(&k.c);
+#pragma unroll
+    for (int h = 0; h < RPL / 2; ++h) {
+        a[2 * h] = fma2(ka.x, b[2 * h], fma2(ka.y, b[2 * h + 1], a[2 * h]));
+        a[2 * h + 1] = fma2(ka.x, b[2 * h + 1], fma2(kb.x, b[2 * h], a[2 * h + 1]));
+        b[2 * h] = fma2(kb.y, a[2 * h], fma2(kc.x, a[2 * h + 1], b[2 * h]));
+        b[2 * h + 1] = fma2(kb.y, a[2 * h + 1], fma2(kc.y, a[2 * h], b[2 * h + 1]));
+    }
+}
+template <int RPL>
+__device__ __forceinline__ void col_rotate(double2 (&a)[RPL], double2 (&b)[RPL], const Coef<double>& k) {
+    const double tr = k.t.x, ti = k.t.y, kr = k.k.x, ki = k.k.y;
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) {
+        a[q].x = fma(-tr, b[q].x, fma(-ti, b[q].y, a[q].x));
+        a[q].y = fma(-tr, b[q].y, fma(ti, b[q].x, a[q].y));
+        b[q].x = fma(kr, a[q].x, fma(-ki, a[q].y, b[q].x));
+        b[q].y = fma(kr, a[q].y, fma(ki, a[q].x, b[q].y));
+    }
+}
+// a += d a
+template <int RPL>
+__device__ __forceinline__ void col_scale(unsigned long long (&a)[RPL], float d) {
+    const unsigned long long dd = pk2(d, d);
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) a[q] = fma2(dd, a[q], a[q]);
+}
+template <int RPL>
+__device__ __forceinline__ void col_scale(double2 (&a)[RPL], double d) {
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) {
+        a[q].x = fma(d, a[q].x, a[q].x);
+        a[q].y = fma(d, a[q].y, a[q].y);
+    }
+}
+// |a|^2 over the warp
+template <int RPL>
+__device__ __forceinline__ float col_norm2(const unsigned long long (&a)[RPL]) {
+    unsigned long long s = 0ull;
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) s = fma2(a[q], a[q], s);
+    const float2 t = upk2(s);
+    return warp_sum(t.x + t.y);
+}
+template <int RPL>
+__device__ __forceinline__ double col_norm2(const double2 (&a)[RPL]) {
+    double s0 = 0, s1 = 0;
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) {
+        s0 = fma(a[q].x, a[q].x, s0);
+        s1 = fma(a[q].y, a[q].y, s1);
+    }
+    return warp_sum(s0 + s1);
+}
+
+// The sums over the warp of B complex values a lane, the p-th to the lanes
+// p (32/B) .. (p + 1)(32/B) - 1.
+template <typename R, int B>
+__device__ __forceinline__ void reduce_pairs(R (&vr)[B], R (&vi)[B], int lane, R& gr, R& gi) {
+    constexpr unsigned kAll = 0xffffffffu;
+    if constexpr (B == 4) {
+        const bool hi = lane & 16;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const R sr = hi ? vr[i] : vr[i + 2], si = hi ? vi[i] : vi[i + 2];
+            const R kr = hi ? vr[i + 2] : vr[i], ki = hi ? vi[i + 2] : vi[i];
+            vr[i] = kr + __shfl_xor_sync(kAll, sr, 16);
+            vi[i] = ki + __shfl_xor_sync(kAll, si, 16);
+        }
+    }
+    if constexpr (B >= 2) {
+        constexpr int o = B == 4 ? 8 : 16;
+        const bool hi = lane & o;
+        const R sr = hi ? vr[0] : vr[1], si = hi ? vi[0] : vi[1];
+        const R kr = hi ? vr[1] : vr[0], ki = hi ? vi[1] : vi[0];
+        vr[0] = kr + __shfl_xor_sync(kAll, sr, o);
+        vi[0] = ki + __shfl_xor_sync(kAll, si, o);
+    }
+#pragma unroll
+    for (int o = 16 / B; o > 0; o >>= 1) {
+        vr[0] += __shfl_xor_sync(kAll, vr[0], o);
+        vi[0] += __shfl_xor_sync(kAll, vi[0], o);
+    }
+    gr = vr[0];
+    gi = vi[0];
+}
+
+// The rotation that diagonalises [[al, g], [conj(g), be]] (al = |a|^2, be = |b|^2,
+// g = a^H b): (tr, ti) = tan(angle) e^{i arg g}, tg = tan(angle) |g| (the norms
+// become al - tg and be + tg), c2 = cos^2, cm1 = cos - 1, sm1 = 1/cos - 1.  In full,
+// a' = cos (a - conj(tau) b) and b' = cos (b + tau a) with tau = (tr, ti); since
+// b + tau a = (1 + |tau|^2) (b + cos^2 tau (a - conj(tau) b)), the second shear has
+// kappa = cos^2 tau and b takes the factor 1/cos.
+// t = 2 |g| sign(d) / (|d| + sqrt(d^2 + 4 |g|^2)), d = be - al: the smaller root
+// of t^2 + (d / |g|) t - 1 = 0, formed without a quotient by |g|.
+template <typename R> struct Rot { R tr, ti, tg, c2, cm1, sm1; };
+
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// 1 / w for w of moderate size: the approximate reciprocal and Newton steps to
+// working precision (a biased quotient in every rotation would add up in the norms)
+__device__ __forceinline__ float rcp_newton(float w) {
+    const float y = rcp_approx(w);
+    return fmaf(y, fmaf(-w, y, 1.0f), y);
+}
+__device__ __forceinline__ double rcp_newton(double w) {
+    double y = (double)rcp_approx((float)w);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) y = fma(y, fma(-w, y, 1.0), y);
+    return y;
+}
+
+__device__ __forceinline__ Rot<float> rotation(float al, float be, float gr, float gi, float g2) {
+    const float d = be - al;
+    const float h = fmaf(d, d, 4.0f * g2);
+    const float root = h * rsqrtf(h);
+    float f = __fdividef(2.0f, fabsf(d) + root);
+    if (d < 0.0f) f = -f;
+    Rot<float> p;
+    p.tr = f * gr;
+    p.ti = f * gi;
+    p.tg = f * g2;
+    const float t2 = f * p.tg;
+    const float q = 1.0f + t2;
+    p.c2 = rcp_newton(q);
+    float c = rsqrt_approx(q);  // refined by one Newton step: c^2 q = 1 to rounding, with no biased residual
+    c = c * fmaf(-0.5f * q * c, c, 1.5f);
+    p.sm1 = t2 * rcp_newton(fmaf(q, c, 1.0f));  // 1/cos = q c
+    p.cm1 = -p.sm1 * c;
+    return p;
+}
+// complex128: tan(angle) e^{i arg g} is worked out in FP32 from values scaled by
+// a power of two (a tangent that is 1e-7 off leaves the pair orthogonal to
+// 1e-7 of its cos, which the next sweep's quadratic convergence does not notice),
+// since the FP64 square root and division cost more than the pair's dot product
+// there; cos is then taken from that same tangent in FP64, so that the rotation
+// is unitary to FP64 rounding.
+__device__ __forceinline__ Rot<double> rotation(double al, double be, double gr, double gi, double) {
+    const double big = fmax(al, be);
+    const int e = (__double2hiint(big) >> 20) & 0x7ff;
+    const int ie = 2046 - e;  // exponent field of 2^(1023 - e)
+    const double s = __hiloint2double((ie < 1 ? 1 : ie) << 20, 0);
+    const double d = be - al;
+    const float df = (float)(d * s), grf = (float)(gr * s), gif = (float)(gi * s);
+    const float g2 = fmaf(grf, grf, gif * gif);
+    const float h = fmaf(df, df, 4.0f * g2);
+    const float root = h > 0.0f ? h * rsqrtf(h) : 0.0f;
+    float f = __fdividef(2.0f, fabsf(df) + root);
+    if (d < 0.0) f = -f;
+    Rot<double> p;
+    p.tr = (double)(f * grf);
+    p.ti = (double)(f * gif);
+    p.tg = fma(p.tr, gr, p.ti * gi);
+    const double t2 = fma(p.tr, p.tr, p.ti * p.ti);
+    const double q = 1.0 + t2;
+    double c = (double)rsqrt_approx((float)q);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) c = c * fma(-0.5 * q * c, c, 1.5);
+    p.c2 = c * c;
+    p.sm1 = t2 * rcp_newton(fma(q, c, 1.0));
+    p.cm1 = -p.sm1 * c;
+    return p;
+}
+// ------------------------------------------------------------ one warp --
+// Columns of a group and rows a lane holds of each: the 2 B columns of a visit
+// take 2 B RPL complex registers (128 32-bit registers at 512 rows complex64,
+// 512 rows complex128 and every size in between down to 128 rows complex128).
+template <typename R, int RPL> struct GroupCols {
+    static constexpr int v = std::is_same<R, float>::value ? (RPL >= 16 ? 2 : 4) : (RPL >= 16 ? 1 : RPL >= 8 ? 2 : 4);
+};
+
+// What a warp carries through a sweep.
+template <typename R> struct Sweep {
+    R tol2, big2;
+    bool big = false;  // this lane's pair was rotated with cos^2 >= big2
+    int rot = 0;       // rotations of this warp
+};
+
+// One round of B disjoint pairs (a[i], y[(i + r) mod B]).  Lane group p holds
+// al, da, fa of column p of a and be, db, fb of column (p + r) mod B of y: true
+// squared norm, scale minus 1, and (complex128) whether the column was rotated
+// in this sweep or the one before.  Pairs of two columns with neither flag set
+// met in the sweep before as the same two vectors and were orthogonal: their
+// dot product is left out (on the FP64 pipe it costs a third of a rotation, and
+// late sweeps are mostly such checks).  Returns the mask of lanes whose pair
+// rotated.
+template <typename R, int RPL, int B, int r>
+__device__ __forceinline__ unsigned round_pairs(entry_t<R> (&a)[B][RPL], entry_t<R> (&y)[B][RPL], R& al, R& da, int& fa,
+                                                R& be, R& db, int& fb, bool pair_ok, Sweep<R>& sw, Coef<R>* tb, int lane) {
+    constexpr bool kSkip = std::is_same<R, double>::value;
+    constexpr int L = 32 / B;
+    const int p = lane / L;
+    R vr[B], vi[B];
+    unsigned need = 0xffffffffu;
+    if constexpr (kSkip) {
+        need = __ballot_sync(0xffffffffu, pair_ok && (fa | fb));
+        if (!need) return 0u;
+    }
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+        vr[i] = 0;
+        vi[i] = 0;
+        if (!kSkip || ((need >> (i * L)) & 1u)) col_dot<RPL>(a[i], y[(i + r) % B], vr[i], vi[i]);
+    }
+    const R wa = (R)1 + da, wb = (R)1 + db;
+    const R ia = rcp_newton(wa), ib = rcp_newton(wb);
+    R gr, gi;
+    reduce_pairs<R, B>(vr, vi, lane, gr, gi);
+    const R sc = wa * wb;
+    gr *= sc;
+    gi *= sc;
+    const R g2 = gr * gr + gi * gi;
+    // al, be >= 0 (a tracked norm that shrinks a lot is recomputed from its
+    // column), so a zero column (g = 0) or a non-finite value fails this test and
+    // is left alone
+    const bool rot = pair_ok && g2 > (sw.tol2 * al) * be;
+    const unsigned m = __ballot_sync(0xffffffffu, rot);
+    if (!m) return 0u;
+    // (no branch: the lanes of pairs that stay compute along and drop the result)
+    sw.big = sw.big || (rot && g2 > (sw.big2 * al) * be);
+    const Rot<R> q = rotation(al, be, gr, gi, g2);
+    const R u = wb * ia, w = wa * ib * q.c2;
+    __syncwarp();  // the warp is done with the coefficients of the round before
+    // short columns: every pair of the round is sheared, a pair that stays by zero
+    // (cheaper than a branch per pair); long ones: only the pairs that rotate
+    constexpr bool kAll = RPL <= 4 && !kSkip;
+    if ((kAll || rot) && (lane & (L - 1)) == 0)
+        tb[p].set(rot ? q.tr * u : (R)0, rot ? q.ti * u : (R)0, rot ? q.tr * w : (R)0, rot ? q.ti * w : (R)0);
+    const R al2 = rot ? al - q.tg : al, be2 = rot ? be + q.tg : be;
+    const R cm1 = rot ? q.cm1 : (R)0, sm1 = rot ? q.sm1 : (R)0;
+    // a norm that lost most of its size (cancellation in the update) is taken from its column
+    const bool shrunk = rot && !(al2 > (R)0.125 * al && be2 > (R)0.125 * be);
+    const bool sa = !(al2 > (R)0.125 * al), sb = !(be2 > (R)0.125 * be);
+    al = al2;
+    be = be2;
+    da = da + fma(da, cm1, cm1);
+    db = db + fma(db, sm1, sm1);
+    if constexpr (kSkip) {
+        fa |= rot ? 2 : 0;
+        fb |= rot ? 2 : 0;
+    }
+    __syncwarp();
+    sw.rot += __popc(m) / L;
+#pragma unroll
+    for (int i = 0; i < B; ++i)
+        if (kAll || ((m >> (i * L)) & 1u)) col_rotate<RPL>(a[i], y[(i + r) % B], tb[i]);
+    if (__any_sync(0xffffffffu, shrunk)) {
+        const unsigned ma = __ballot_sync(0xffffffffu, shrunk && sa), mb = __ballot_sync(0xffffffffu, shrunk && sb);
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+            if ((ma >> (i * L)) & 1u) {
+                const R n2 = col_norm2<RPL>(a[i]);
+                if (p == i) al = n2 * ((R)1 + da) * ((R)1 + da);
+            }
+            if ((mb >> (i * L)) & 1u) {
+                const R n2 = col_norm2<RPL>(y[(i + r) % B]);
+                if (p == i) be = n2 * ((R)1 + db) * ((R)1 + db);
+            }
+        }
+    }
+    return m;
+}
+
+template <typename R, int RPL, int B, int r>
+__device__ __forceinline__ unsigned visit_rounds(entry_t<R> (&a)[B][RPL], entry_t<R> (&y)[B][RPL], R& al, R& da, int& fa,
+                                                 R& be, R& db, int& fb, Sweep<R>& sw, Coef<R>* tb, int lane) {
+    if constexpr (r == B) {
+        return 0u;
+    } else {
+        unsigned m = round_pairs<R, RPL, B, r>(a, y, al, da, fa, be, db, fb, true, sw, tb, lane);
+        if constexpr (B > 1) {  // lane group p goes on to column (p + r + 1) mod B of y
+            constexpr int L = 32 / B;
+            const int src = (lane + L) & 31;
+            be = __shfl_sync(0xffffffffu, be, src);
+            db = __shfl_sync(0xffffffffu, db, src);
+            if constexpr (std::is_same<R, double>::value) fb = __shfl_sync(0xffffffffu, fb, src);
+        }
+        return m | visit_rounds<R, RPL, B, r + 1>(a, y, al, da, fa, be, db, fb, sw, tb, lane);
+    }
+}
+
+// Multiply the scales out: column i of a by 1 + (the da of lane group i).
+template <typename R, int RPL, int B>
+__device__ __forceinline__ void apply_scales(entry_t<R> (&a)[B][RPL], R& da) {
+#pragma unroll
+    for (int i = 0; i < B; ++i) col_scale<RPL>(a[i], __shfl_sync(0xffffffffu, da, i * (32 / B)));
+    da = 0;
+}
+
+// The pairs inside a group.
+template <typename R, int RPL, int B>
+__device__ __forceinline__ bool inner_pairs(entry_t<R> (&a)[B][RPL], R& al, R& da, int& fa, Sweep<R>& sw, Coef<R>* tb,
+                                            int lane) {
+    if constexpr (B == 1) {
+        return false;
+    } else {
+        // (B = 2) one pair; (B = 4) three rounds of two pairs: (0,1)(2,3), (0,2)(1,3), (0,3)(1,2).
+        // Taken through round_pairs with B/2 columns a side; lane groups of B/2 pairs.
+        constexpr int H = B / 2, L = 32 / B, LH = 32 / H;
+        const int ph = lane / LH;
+        unsigned any = 0u;
+        auto one = [&](auto rc) {
+            constexpr int k = decltype(rc)::value;
+            // columns x(q), z(q) of pair q
+            constexpr int x0 = 0, x1 = k == 0 ? 2 : 1;
+            constexpr int z0 = k + 1, z1 = k == 0 ? 3 : k == 1 ? 3 : 2;
+            entry_t<R> x[H][RPL], z[H][RPL];
+#pragma unroll
+            for (int q = 0; q < RPL; ++q) {
+                x[0][q] = a[x0][q];
+                z[0][q] = a[z0][q];
+                if constexpr (H == 2) {
+                    x[1][q] = a[x1][q];
+                    z[1][q] = a[z1][q];
+                }
+            }
+            const int sx = (ph == 0 ? x0 : x1) * L, sz = (ph == 0 ? z0 : z1) * L;
+            R ax = __shfl_sync(0xffffffffu, al, sx), az = __shfl_sync(0xffffffffu, al, sz);
+            R dx = __shfl_sync(0xffffffffu, da, sx), dz = __shfl_sync(0xffffffffu, da, sz);
+            int fx = __shfl_sync(0xffffffffu, fa, sx), fz = __shfl_sync(0xffffffffu, fa, sz);
+            const unsigned m = round_pairs<R, RPL, H, 0>(x, z, ax, dx, fx, az, dz, fz, true, sw, tb, lane);
+            if (m) {
+                any |= m;
+#pragma unroll
+                for (int q = 0; q < RPL; ++q) {
+                    a[x0][q] = x[0][q];
+                    a[z0][q] = z[0][q];
+                    if constexpr (H == 2) {
+                        a[x1][q] = x[1][q];
+                        a[z1][q] = z[1][q];
+                    }
+                }
+                // back to one lane group per column
+                const int p = lane / L;
+                const bool is_x = p == x0 || (H == 2 && p == x1);
+                const int pair = (p == x0 || p == z0) ? 0 : 1;
+                const int src = pair * LH;
+                const R bx = __shfl_sync(0xffffffffu, ax, src), bz = __shfl_sync(0xffffffffu, az, src);
+                const R ex = __shfl_sync(0xffffffffu, dx, src), ez = __shfl_sync(0xffffffffu, dz, src);
+                const int gx = __shfl_sync(0xffffffffu, fx, src), gz = __shfl_sync(0xffffffffu, fz, src);
+                al = is_x ? bx : bz;
+                da = is_x ? ex : ez;
+                fa = is_x ? gx : gz;
+            }
+        };
+        one(std::integral_constant<int, 0>{});
+        if constexpr (B == 4) {
+            one(std::integral_constant<int, 1>{});
+            one(std::integral_constant<int, 2>{});
+        }
+        return any != 0u;
+    }
+}
+
+// ------------------------------------------------------------- one CTA --
+constexpr int kMaxCols = 2 * PTEBD_CHI_LIMIT;  // 512
+constexpr int kMaxSlots = 32;
+constexpr int kMaxWarps = 16;
+constexpr double kScaleMax = 1.0 / 64;
+constexpr int kLag = 6;  // positions between a group's way back to W and the reuse of its slot
+
+// Tables of a CTA, ahead of the columns in shared memory.
+template <typename R> struct Tables {
+    uint64_t full[kMaxSlots];      // TMA loads of the slots
+    Coef<R> tb[kMaxWarps][4];      // rotation coefficients of a round, per warp
+    R nrm[kMaxCols];               // squared column norms (by column)
+    R pnrm[kMaxCols];              // the same in sweep order
+    R scl[kMaxCols];               // scales minus 1 (by column)
+    R pscl[kMaxCols];              // the same in sweep order
+    uint32_t key[kMaxCols];        // sort keys
+    int cperm[kMaxCols];           // sweep order -> column
+    int prog[kMaxCols];            // I groups that have met group j (in this sweep); j + 1 once it is taken itself
+    int dirty[kMaxCols];           // streaming: group j was rotated since it was last fetched
+    unsigned char flag[kMaxCols];  // complex128, by column: rotated in the sweep before
+    unsigned char pflag[kMaxCols]; // by position: bit 0 the sweep before, bit 1 this one
+    int rotations, abort, max_exp, big;
+    int fetch_e, fetch_k, fetch_g, fetch_slot;  // streaming: the next position to fetch, its row, group and slot
+};
+
+// Smallest power of two >= 1 + the table size, so that the columns start 128-byte aligned.
+template <typename R> constexpr size_t table_bytes() { return (sizeof(Tables<R>) + 127) / 128 * 128; }
+
+// Dynamic shared memory: the tables and `column_area` bytes of columns.
+constexpr int kSmemMax = 227 * 1024;
+template <typename R> int column_area(int ldw, bool half) {
+    // (a column of zeros beside the matrix; at least 64 rows a column on complex64)
+    const size_t all = (size_t)(ldw + 1) * (ldw < 64 ? 64 : ldw) * sizeof(cx_t<R>);
+    const size_t most = (half ? kSmemMax / 2 - 1024 : kSmemMax) - table_bytes<R>();
+    return (int)(all < most ? all : most);
+}
+// Compute warps: no more than groups of the widest matrix, at most `most`.
+inline int warps_for(int ldw, bool half, int most) {
+    const int w = ldw / 4 < most ? ldw / 4 : most;
+    return half && w > 4 ? 4 : w;
+}
+
+template <typename R, int RPL, bool RES>
+__device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int rows, int cols, int j_slot,
+                                         int area, Tables<R>* T, cx_t<R>* cbuf) {
+    const bool wait_test = A.wait_test != 0;
+    const int chi_max = A.chi_max, max_sweeps = A.max_sweeps;
+    using C = cx_t<R>;
+    constexpr int B = GroupCols<R, RPL>::v;
+    constexpr int L = 32 / B;
+    constexpr int mpad = 32 * RPL;  // rows per column in shared memory
+    constexpr bool kSkip = std::is_same<R, double>::value;
+    constexpr bool kSplit = std::is_same<R, float>::value;
+    const int ldw = A.ldw;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nwc = blockDim.x >> 5;
+    const int G = (cols + B - 1) / B;
+    const int S = RES ? G : min(kMaxSlots, (int)((area - mpad * sizeof(C)) / (B * mpad * sizeof(C))));  // slots
+    C* const zeros = cbuf + (RES ? cols : S * B) * mpad;
+    const uint32_t col_bytes = (uint32_t)(rows * sizeof(C));
+    volatile int* abort_flag = &T->abort;
+
+    // columns in shared memory start as zeros (rows beyond `rows` stay zero)
+    for (int e = tid; e < (RES ? cols + 1 : S * B + 1) * mpad; e += blockDim.x) cbuf[e] = cmake<C>(0, 0);
+    for (int c = tid; c < cols; c += blockDim.x) {
+        T->scl[c] = 0;
+        if constexpr (kSkip) T->flag[c] = 1;  // sweep 0 checks every pair
+    }
+    fence_async_smem();
+    __syncthreads();
+
+    // squared norms of the columns (exact); with `first`, the exponent of the
+    // largest |entry| is gathered, and the columns are read from W (RES) and put
+    // into the pair-split layout (complex64)
+    auto column = [&](int c) -> C* { return RES ? cbuf + (size_t)c * mpad : W + (size_t)c * ldw; };
+    auto norm_pass = [&](bool first) {
+        R mx = 0;
+        for (int c = warp; c < cols; c += nwc) {
+            R s0 = 0, s1 = 0;
+            const C* src = first ? W + (size_t)c * ldw : column(c);
+            C* dst = column(c);
+            if constexpr (kSplit) {
+                for (int g = lane; g < rows / 2; g += 32) {
+                    const float4 v = reinterpret_cast<const float4*>(src)[g];
+                    s0 = fma(v.x, v.x, s0); s1 = fma(v.y, v.y, s1);
+                    s0 = fma(v.z, v.z, s0); s1 = fma(v.w, v.w, s1);
+                    if (first) {
+                        mx = fmax(mx, fmax(fmax(fabs(v.x), fabs(v.y)), fmax(fabs(v.z), fabs(v.w))));
+                        reinterpret_cast<float4*>(dst)[g] = make_float4(v.x, v.z, v.y, v.w);
+                    }
+                }
+            } else {
+                for (int r = lane; r < rows; r += 32) {
+                    const C v = src[r];
+                    s0 = fma(v.x, v.x, s0);
+                    s1 = fma(v.y, v.y, s1);
+                    if (first) {
+                        mx = fmax(mx, fmax(fabs(v.x), fabs(v.y)));
+                        if constexpr (RES) dst[r] = v;
+                    }
+                }
+            }
+            const R w = (R)1 + T->scl[c], s2 = warp_sum(s0 + s1) * w * w;
+            if (lane == 0) T->nrm[c] = s2;
+        }
+        if (first) {
+            mx = warp_max(mx);
+            if (lane == 0) atomicMax(&T->max_exp, exp_key<R>(mx));
+            if (!RES) fence_async_global();  // the sweeps read W through TMA as well
+        }
+    };
+
+    const R tol = (R)(Eps<R>::k * sqrt((double)rows) * Eps<R>::u);
+    Sweep<R> sw;
+    sw.tol2 = tol * tol;
+    sw.big2 = (R)Eps<R>::early * sw.tol2;
+    const bool polish = A.polish && Eps<R>::polish > 0.0;
+    bool polishing = false;  // the last sweep, with the tighter threshold
+    bool converged = false;
+    long long rot_total = 0;
+    int scale_e = 0;
+    int streamed = 0;  // groups streamed in the sweeps before this one (the same on every warp)
+    int sweep = 0;
+    Coef<R>* tb = T->tb[warp];
+
+    for (sweep = 0; sweep < max_sweeps; ++sweep) {
+        norm_pass(sweep == 0);
+        __syncthreads();
+        if (sweep == 0) {
+            // Range guard.  Squared norms and |a^H b|^2 are formed in R: with entries of
+            // 2^range_e and more they can overflow (and with tiny entries underflow),
+            // which turns a rotation into a plain scaling of the pair.  Such a matrix is
+            // scaled by 2^-e, exactly, so that its largest entry lies in [1, 2), and
+            // scaled back after the sweeps: a power-of-two scaling commutes with every
+            // rounding of the sweeps, so the result equals that of an unbounded exponent
+            // range.
+            const int ex = T->max_exp - kExpOffset;  // 2^ex <= max |entry| < 2^(ex + 1)
+            if (T->max_exp > 0 && (ex >= Eps<R>::range_e || ex < -Eps<R>::range_e)) {
+                scale_e = ex;
+                const R f = ldexp((R)1, -scale_e);
+                for (int c = warp; c < cols; c += nwc) {
+                    C* col = column(c);
+                    for (int r = lane; r < rows; r += 32) {
+                        C v = col[r];
+                        v.x *= f; v.y *= f;
+                        col[r] = v;
+                    }
+                }
+                if (!RES) fence_async_global();
+                __syncthreads();
+                norm_pass(false);
+                __syncthreads();
+            }
+        }
+        // sweep order: columns by decreasing norm, ties by index (ranks counted from
+        // integer keys, so that any values give a permutation)
+        for (int c = tid; c < cols; c += blockDim.x)
+            T->key[c] = __float_as_uint((float)T->nrm[c]) & 0x7fffffffu;
+        for (int g = tid; g < G; g += blockDim.x) { T->prog[g] = 0; T->dirty[g] = 0; }
+        __syncthreads();
+        for (int c = tid; c < cols; c += blockDim.x) {
+            const uint32_t mine = T->key[c];
+            int rank = 0;
+            for (int q = 0; q < cols; ++q) {
+                const uint32_t k = T->key[q];
+                rank += (k > mine || (k == mine && q < c)) ? 1 : 0;
+            }
+            T->cperm[rank] = c;
+            T->pnrm[rank] = T->nrm[c];
+            T->pscl[rank] = T->scl[c];
+            if constexpr (kSkip) T->pflag[rank] = T->flag[c];
+        }
+        __syncthreads();
+
+        // the polish sweep leaves pairs of two columns beyond chi_max (in the sweep
+        // order, by decreasing norm) alone: they are dropped together, a rotation
+        // between them changes no kept column and keeps their summed weight
+        const int GI = polishing && chi_max > 0 ? min(G, (chi_max + B - 1) / B) : G;
+        {
+            bool ok = true;
+            const int p = lane / L;
+            // Streaming: position in the sweep's stream of groups (rows of I groups one after
+            // the other, each from its first group k0 to G - 1), its slot and the slot's phase.
+            int rel = 0, slot = 0;
+            uint32_t phase = 0;
+            if constexpr (!RES) { slot = streamed % S; phase = (uint32_t)(streamed / S) & 1u; }
+            auto advance = [&](int d) {
+                if constexpr (!RES) {
+                    rel += d;
+                    slot += d;
+                    while (slot >= S) { slot -= S; phase ^= 1u; }
+                }
+            };
+            // The last warp fetches the groups in the order the warps meet them.  `done`: the
+            // last position it has met; every position it meets has its bulk group (empty if
+            // nothing was stored), so that "all but the last kLag groups complete" says that
+            // the positions up to done - kLag are back in W and their slots free.
+            auto pump = [&](int done, bool drain) {
+                if (lane == 0) {
+                    int e = T->fetch_e, k0 = T->fetch_k, g = T->fetch_g, sl = T->fetch_slot;
+                    if (drain) bulk_wait<0>(); else bulk_wait<kLag>();
+                    const int free_to = drain ? done : done - kLag;
+                    fence_async_smem();
+                    while (k0 < GI && e - S <= free_to && (k0 == 0 || e - (G - k0) <= free_to)) {
+                        const int nc = min(B, cols - g * B);
+                        mbar_expect_tx(&T->full[sl], (uint32_t)nc * col_bytes);
+                        for (int i = 0; i < nc; ++i)
+                            bulk_g2s(cbuf + ((size_t)sl * B + i) * mpad, W + (size_t)T->cperm[g * B + i] * ldw,
+                                     col_bytes, &T->full[sl]);
+                        ++e;
+                        if (++sl == S) sl = 0;
+                        if (++g == G) { k0 += nwc; g = k0; }
+                    }
+                    T->fetch_e = e; T->fetch_k = k0; T->fetch_g = g; T->fetch_slot = sl;
+                }
+                __syncwarp();
+            };
+            // What is left to fetch once the last warp has no I group of its own (the last row
+            // of a polish sweep): as the groups before get through.
+            auto pump_rest = [&]() -> bool {
+                bool fine = true;
+                while (fine && T->fetch_k < GI) {
+                    const int k0 = T->fetch_k, e = T->fetch_e;
+                    int tj = e - S, tk = 0;  // the group in the slot
+                    while (tj >= G - tk) { tj -= G - tk; tk += nwc; }
+                    tj += tk;
+                    fine = (e < S || counter_wait(&T->prog[tj], min(tj + 1, min(tk + nwc, GI)), abort_flag)) &&
+                           (k0 == 0 || counter_wait(&T->prog[T->fetch_g], k0, abort_flag));
+                    fine = __all_sync(0xffffffffu, fine);
+                    if (fine) pump(max(e - S, e - (G - k0)), true);
+                }
+                return fine;
+            };
+            const bool fetcher = !RES && warp == nwc - 1;
+            if (fetcher) {
+                if (lane == 0) { T->fetch_e = T->fetch_k = T->fetch_g = 0; T->fetch_slot = slot; }
+                __syncwarp();
+                pump(-1, true);
+            }
+            for (int k0 = 0; k0 < GI && ok; k0 += nwc) {
+                const int I = k0 + warp;
+                if (I >= GI) break;
+                const bool last = !RES && I == min(k0 + nwc, GI) - 1;  // the last warp of the row
+                // Group g has met every I before this one (streaming, the first warp of a row: it
+                // has been fetched).  The same answer on every lane: they read one address in
+                // one instruction, and a wait that did not succeed at once ends in a vote.
+                auto ready = [&](int g) -> bool {
+                    if (RES ? I == 0 : warp == 0) {
+                        if constexpr (!RES)
+                            if (!mbar_try_wait(&T->full[slot], phase))
+                                return __all_sync(0xffffffffu, mbar_wait(&T->full[slot], phase, abort_flag));
+                        return true;
+                    }
+                    const bool test = wait_test && sweep == 0 && I == 1 && g == 1;
+                    if (counter_acquire(&T->prog[g]) >= I && !test) return true;
+                    return __all_sync(0xffffffffu, counter_wait(&T->prog[g], test ? 0x7fffffff : I, abort_flag,
+                                                                test ? (1ll << 20) : kWaitLimit));
+                };
+                // address of column i of group g in shared memory
+                auto sm_col = [&](int g, int i) -> C* {
+                    const int pos = g * B + i;  // (columns missing from the last group: a column of zeros)
+                    if (pos >= cols) return zeros;
+                    if constexpr (RES) return cbuf + T->cperm[pos] * mpad;
+                    return cbuf + (slot * B + i) * mpad;
+                };
+                advance(warp);
+                if (!ready(I)) { ok = false; break; }
+                entry_t<R> a[B][RPL];
+#pragma unroll
+                for (int i = 0; i < B; ++i) col_load<RPL>(a[i], sm_col(I, i), lane);
+                const bool ip = I * B + p < cols;
+                R al = ip ? T->pnrm[I * B + p] : (R)0, da = ip ? T->pscl[I * B + p] : (R)0;
+                int fa = 0;
+                if constexpr (kSkip) fa = ip ? T->pflag[I * B + p] : 0;
+                bool changed = !RES && T->dirty[I] != 0;
+                __syncwarp();
+                if (lane == 0) counter_release(&T->prog[I], I + 1);
+                if (fetcher) {
+                    if (lane == 0)
+                        for (int q = 0; q < nwc; ++q) bulk_commit();
+                }
+                changed = inner_pairs<R, RPL, B>(a, al, da, fa, sw, tb, lane) || changed;
+                for (int J = I + 1; J < G; ++J) {
+                    advance(1);
+                    if (!ready(J)) { ok = false; break; }
+                    const bool jp = J * B + p < cols;
+                    R be = jp ? T->pnrm[J * B + p] : (R)0, db = jp ? T->pscl[J * B + p] : (R)0;
+                    int fb = 0;
+                    if constexpr (kSkip) fb = jp ? T->pflag[J * B + p] : 0;
+                    bool store = last && T->dirty[J] != 0;
+                    if (!kSkip || __any_sync(0xffffffffu, fa | fb)) {
+                        entry_t<R> y[B][RPL];
+#pragma unroll
+                        for (int i = 0; i < B; ++i) col_load<RPL>(y[i], sm_col(J, i), lane);
+                        if (visit_rounds<R, RPL, B, 0>(a, y, al, da, fa, be, db, fb, sw, tb, lane)) {
+                            changed = true;
+                            store = last;
+                            if (__any_sync(0xffffffffu, fabs(db) > (R)kScaleMax)) apply_scales<R, RPL, B>(y, db);
+                            if (__any_sync(0xffffffffu, fabs(da) > (R)kScaleMax)) apply_scales<R, RPL, B>(a, da);
+                            if (jp && (lane & (L - 1)) == 0) {
+                                T->pnrm[J * B + p] = be;
+                                T->pscl[J * B + p] = db;
+                                if constexpr (kSkip) T->pflag[J * B + p] = (unsigned char)fb;
+                            }
+#pragma unroll
+                            for (int i = 0; i < B; ++i)
+                                if (J * B + i < cols) col_store<RPL>(y[i], sm_col(J, i), lane, mpad);
+                            if constexpr (!RES)
+                                if (!last && lane == 0) T->dirty[J] = 1;
+                        }
+                    }
+                    __syncwarp();
+                    if constexpr (!RES) {
+                        if (last) {  // a changed group goes back to W
+                            if (lane == 0) {
+                                if (store) {
+                                    T->dirty[J] = 0;
+                                    fence_async_smem();
+                                    const int nc = min(B, cols - J * B);
+                                    for (int i = 0; i < nc; ++i)
+                                        bulk_s2g(W + (size_t)T->cperm[J * B + i] * ldw, sm_col(J, i), col_bytes);
+                                }
+                                bulk_commit();
+                                if (!fetcher) bulk_wait<0>();  // another warp refills the slot
+                            }
+                            __syncwarp();
+                        }
+                    }
+                    if (lane == 0) counter_release(&T->prog[J], I + 1);
+                    if (fetcher) pump(rel, false);
+                }
+                if (!ok) break;
+                if (changed) {
+                    if (ip && (lane & (L - 1)) == 0) T->pscl[I * B + p] = da;
+#pragma unroll
+                    for (int i = 0; i < B; ++i)
+                        if (I * B + i < cols) {
+                            if constexpr (RES) col_store<RPL>(a[i], sm_col(I, i), lane, mpad);
+                            else col_store<RPL>(a[i], W + (size_t)T->cperm[I * B + i] * ldw, lane, rows);
+                        }
+                    if constexpr (kSkip)
+                        if (ip && (lane & (L - 1)) == 0) T->pflag[I * B + p] = (unsigned char)fa;
+                }
+                if (fetcher) pump(rel, true);  // rows shorter than the ring wait for all that was stored
+                advance(1);
+            }
+            if constexpr (!RES) {
+                if (ok && fetcher) ok = pump_rest();
+                bulk_wait<0>();
+                fence_async_global();  // the next sweep reads W through TMA and through plain loads
+            }
+            if (!ok) T->abort = 1;
+        }
+        // groups streamed in this sweep
+        int streamed_now = 0;
+        if constexpr (!RES)
+            for (int k0 = 0; k0 < GI; k0 += nwc) streamed_now += G - k0;
+        streamed += streamed_now;
+        if (lane == 0 && sw.rot) atomicAdd(&T->rotations, sw.rot);
+        if (sw.big) T->big = 1;
+        sw.rot = 0;
+        sw.big = false;
+        __syncthreads();
+        if (T->abort) {
+            // A wait ran out: wait (bounded) for the fetches still in flight and latch the
+            // error.  If one still has not landed, the CTA has to return with it in flight
+            // (nothing can cancel a bulk copy, and waiting on would hang the GPU):
+            // DERR_DRAIN marks the state unusable until it is re-created.
+            if (tid == 0) {
+                bool drained = true;
+                if constexpr (!RES) {
+                    const int n = (streamed - streamed_now) + T->fetch_e;  // groups fetched, over all sweeps
+                    for (int e = max(0, n - S); e < n; ++e)
+                        if (!mbar_wait(&T->full[e % S], (uint32_t)(e / S) & 1u, nullptr)) drained = false;
+                }
+                atomicOr(A.err, drained ? DERR_TIMEOUT : (DERR_TIMEOUT | DERR_DRAIN));
+            }
+            __syncthreads();
+            return;
+        }
+        const int rot = T->rotations;
+        const bool small = Eps<R>::early > 0.0 && T->big == 0;
+        rot_total += rot;
+        for (int q = tid; q < cols; q += blockDim.x) {
+            T->scl[T->cperm[q]] = T->pscl[q];
+            if constexpr (kSkip) T->flag[T->cperm[q]] = T->pflag[q] >> 1;
+        }
+        __syncthreads();
+        if (tid == 0) { T->rotations = 0; T->big = 0; }
+        if (polishing) { converged = true; ++sweep; break; }
+        if (rot == 0 || small) {
+            if (polish) {
+                polishing = true;
+                const R pt = (R)(Eps<R>::polish * sqrt((double)rows) * Eps<R>::u);
+                sw.tol2 = pt * pt;
+                continue;
+            }
+            converged = true;
+            ++sweep;
+            break;
+        }
+    }
+    __syncthreads();
+    if (!converged && tid == 0) atomicOr(A.err, DERR_NOT_CONVERGED);
+    if (tid == 0) {
+        const unsigned long long visits = (unsigned long long)sweep * (unsigned long long)(cols * (cols - 1) / 2) *
+                                          (unsigned long long)rows;
+        A.slot_sweeps[j_slot] = sweep;
+        if (A.refine) {  // the FP64 resolution of a complex64 state, counted apart
+            atomicAdd(&A.work[8], 1ull);
+            atomicAdd(&A.work[9], visits);
+        } else {
+            atomicAdd(&A.work[0], visits);
+            atomicAdd(&A.work[2], (unsigned long long)rot_total);
+            atomicAdd(&A.work[3], (unsigned long long)sweep);
+            atomicAdd(&A.work[4], 1ull);
+            if (A.mode == 1) {  // tSU factors, counted apart as well
+                atomicAdd(&A.work[5], visits);
+                atomicAdd(&A.work[6], (unsigned long long)sweep);
+                atomicAdd(&A.work[7], 1ull);
+            }
+        }
+    }
+    // FP64 column norms = singular values; the columns' scales are multiplied out, the
+    // range guard's scaling is undone and the pair-split layout turned back into plain
+    // complex columns
+    double* nrm = A.norms + (size_t)j_slot * ldw;
+    const R unscale = ldexp((R)1, scale_e);
+    for (int c = warp; c < cols; c += nwc) {
+        double acc = 0.0;
+        const C* src = column(c);
+        C* dst = W + (size_t)c * ldw;
+        const double w = 1.0 + (double)T->scl[c];
+        const R f = (R)w * unscale;
+        if constexpr (kSplit) {
+            for (int g = lane; g < rows / 2; g += 32) {
+                float4 v = reinterpret_cast<const float4*>(src)[g];
+                acc = fma((double)v.x, (double)v.x, acc);
+                acc = fma((double)v.z, (double)v.z, acc);
+                acc = fma((double)v.y, (double)v.y, acc);
+                acc = fma((double)v.w, (double)v.w, acc);
+                v.x *= f; v.y *= f; v.z *= f; v.w *= f;
+                reinterpret_cast<float4*>(dst)[g] = make_float4(v.x, v.z, v.y, v.w);
+            }
+        } else {
+            for (int r = lane; r < rows; r += 32) {
+                C v = src[r];
+                acc = fma((double)v.x, (double)v.x, acc);
+                acc = fma((double)v.y, (double)v.y, acc);
+                v.x *= f; v.y *= f;
+                dst[r] = v;
+            }
+        }
+        acc = warp_sum(acc);
+        if (lane == 0) {
+            const double s = ldexp(sqrt(acc) * w, scale_e);
+            if (!isfinite(s)) atomicOr(A.err, DERR_NONFINITE);
+            nrm[c] = s;
+        }
+    }
+}
+
+// Prologue of the kernels: which matrix, its size, the tables.
+template <typename R> struct Start {
+    int rows, cols, area;
+    cx_t<R>* W;
+    Tables<R>* T;
+    cx_t<R>* cbuf;
+    bool go;
+};
+template <typename R>
+__device__ __forceinline__ Start<R> start(const LayerArgs<R>& A, int area, unsigned char* smem) {
+    Start<R> s;
+    const int32_t* d = A.dims + blockIdx.x * kDims;
+    s.go = !(A.refine == 1 && d[D_REFINE] != 1);  // the FP64 resolution runs only undecided bonds
+    if (!s.go) return s;
+    s.rows = A.pass == 1 ? 2 * d[D_CL] : d[D_ROWS];
+    s.cols = A.pass == 1 ? d[D_CM] : d[D_COLS];
+    s.area = area;
+    s.W = A.w + (size_t)blockIdx.x * A.ldw * A.ldw;
+    s.T = reinterpret_cast<Tables<R>*>(smem);
+    s.cbuf = reinterpret_cast<cx_t<R>*>(smem + table_bytes<R>());
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kMaxSlots; ++i) mbar_init(&s.T->full[i], 1);
+        mbar_init_fence();
+        s.T->rotations = 0; s.T->abort = 0; s.T->max_exp = 0; s.T->big = 0; s.T->fetch_e = 0;
+    }
+    return s;
+}
+
+// Columns that fit in the area stay there; `RPL` 16 never does.
+template <typename R, int RPL>
+__device__ __forceinline__ void run_body(const LayerArgs<R>& A, const Start<R>& s) {
+    const size_t need = (size_t)(s.cols + 1) * 32 * RPL * sizeof(cx_t<R>);
+    if (need <= (size_t)s.area)
+        jacobi_body<R, RPL, true>(A, s.W, s.rows, s.cols, blockIdx.x, s.area, s.T, s.cbuf);
+    else
+        jacobi_body<R, RPL, false>(A, s.W, s.rows, s.cols, blockIdx.x, s.area, s.T, s.cbuf);
+}
+
+}  // namespace jac
+}  // namespace ptebd
