@@ -110,7 +110,9 @@ Layout make_layout(const ptebd_config& cfg) {
     L.off_err = o; o = align256(o + sizeof(uint32_t));
     L.off_gates = o; o = align256(o + nb * 32 * sizeof(double));
     L.off_bonds = o; o = align256(o + 3 * nb * sizeof(int32_t));
-    L.off_scratch = o; o = align256(o + 8 * chip * chip * sizeof(double2) + 8 * sizeof(double));
+    L.off_scratch = o;
+    o = align256(o + kScratch * chip * chip * sizeof(double2) + 16 * sizeof(double2) + 2 * sizeof(double) +
+                 (N + 2) * sizeof(unsigned long long));
     L.off_partials = o; o = align256(o + (size_t)kMaxChunks * 4 * sizeof(double));
     L.state_bytes = o;
     const size_t ldw = (size_t)L.ldw;
@@ -665,180 +667,218 @@ std::vector<int32_t> host_chi(ptebd_state* st, int* rc) {
 }
 
 // ------------------------------------------------------------ contraction --
+// Scratch of a contraction (in the state's buffer).
 struct Chain {
-    ptebd_state* st;       // owns the scratch and the stream
-    double2* mat[8];
-    double* logacc;
+    double2* mat[kScratch];
+    double2* out;                 // up to 16 overlaps
+    double* exponent;             // the power of two taken out of them
+    unsigned long long* largest;  // largest modulus of each step's environment, N + 2 of them
 };
 
 Chain chain_of(ptebd_state* st) {
     Chain c;
-    c.st = st;
     const size_t chip = (size_t)st->L.chip;
     double2* base = at<double2>(st->mem, st->L.off_scratch);
-    for (int i = 0; i < 8; ++i) c.mat[i] = base + (size_t)i * chip * chip;
-    c.logacc = reinterpret_cast<double*>(base + 8 * chip * chip);
+    for (int i = 0; i < kScratch; ++i) c.mat[i] = base + (size_t)i * chip * chip;
+    c.out = base + (size_t)kScratch * chip * chip;
+    c.exponent = reinterpret_cast<double*>(c.out + 16);
+    c.largest = reinterpret_cast<unsigned long long*>(c.exponent + 2);
     return c;
 }
 
-template <typename TB>
-const TB* gamma_ptr(ptebd_state* st, int site, int sigma) {
-    const size_t chip = (size_t)st->L.chip;
-    return reinterpret_cast<const TB*>(st->mem + st->L.off_gamma) + ((size_t)site * 2 + sigma) * chip * chip;
-}
 const double* lam_ptr(ptebd_state* st, int bond) {  // bond in -1..N-1
     return at<double>(st->mem, st->L.off_lam) + (size_t)(bond + 1) * st->L.chip;
 }
-
-// Generic GEMM dispatch on the precisions of the two operands.
-int gemm(ptebd_state* owner, int m, int n, int k, double2 alpha, const void* A, bool a64, int lda, int opA,
-         const void* B, bool b64, int ldb, const double* colscale, double2 beta, double2* Cm, int ldc,
-         const double* rowscale) {
-    cudaError_t e;
-    cudaStream_t s = owner->stream;
-    if (a64 && b64)
-        e = launch_zgemm<double2, double2>(m, n, k, alpha, (const double2*)A, lda, opA, (const double2*)B, ldb,
-                                           colscale, beta, Cm, ldc, rowscale, s);
-    else if (a64)
-        e = launch_zgemm<double2, float2>(m, n, k, alpha, (const double2*)A, lda, opA, (const float2*)B, ldb,
-                                          colscale, beta, Cm, ldc, rowscale, s);
-    else if (b64)
-        e = launch_zgemm<float2, double2>(m, n, k, alpha, (const float2*)A, lda, opA, (const double2*)B, ldb,
-                                          colscale, beta, Cm, ldc, rowscale, s);
-    else
-        e = launch_zgemm<float2, float2>(m, n, k, alpha, (const float2*)A, lda, opA, (const float2*)B, ldb,
-                                         colscale, beta, Cm, ldc, rowscale, s);
-    if (e != cudaSuccess) return set_err(owner, PTEBD_ERR_CUDA, "gemm launch failed: %s", cudaGetErrorString(e));
-    return PTEBD_OK;
-}
-
-const void* gptr(ptebd_state* st, int site, int sigma) {
-    return st->cfg.precision == PTEBD_FP64 ? (const void*)gamma_ptr<double2>(st, site, sigma)
-                                           : (const void*)gamma_ptr<float2>(st, site, sigma);
-}
 bool is64(ptebd_state* st) { return st->cfg.precision == PTEBD_FP64; }
+const void* gptr(ptebd_state* st, int site, int sigma) {
+    const size_t chip = (size_t)st->L.chip;
+    return st->mem + st->L.off_gamma + ((size_t)site * 2 + sigma) * chip * chip * st->L.elem;
+}
 
-const double2 ONE = {1.0, 0.0};
-const double2 ZERO = {0.0, 0.0};
+// C = op_a(A) op_b(B), one segment
+Zmm zmm(int m, int n, int k, const void* a, bool a32, int lda, int op_a, const void* b, bool b32, int ldb, int op_b,
+        double2* c, int ldc) {
+    Zmm q{};
+    q.a[0] = a; q.b[0] = b; q.c = c;
+    q.m = m; q.n = n; q.k = k; q.segments = 1;
+    q.lda = lda; q.ldb = ldb; q.ldc = ldc;
+    q.op_a = op_a; q.op_b = op_b;
+    q.a32 = a32; q.b32 = b32;
+    return q;
+}
 
-// <a| O |b> with O = identity everywhere except a one-site op on `site1` or a
-// two-site op on (site2, site2+1) (both -1 for none).  op is row-major complex.
-int contract(ptebd_state* a, ptebd_state* b, int site1, int site2, const double* op, double out[2]) {
-    ptebd_state* own = a;
-    Chain ch = chain_of(own);
+// Adds to the two batches of a step (the T_x, then the sum over x) what takes the left
+// environment `e` of site s to that of site s + 1, `en`; `seen` / `next`: the largest
+// moduli of the two.
+void left_step(ptebd_state* a, ptebd_state* b, const std::vector<int32_t>& ca, const std::vector<int32_t>& cb, int s,
+               const double2* e, double2* en, double2* t0, double2* t1, const unsigned long long* seen,
+               unsigned long long* next, ZmmBatch& first, int& nf, ZmmBatch& second, int& ns) {
+    const int ld = a->L.chip, al = ca[s], ar = ca[s + 1], bl = cb[s], br = cb[s + 1];
+    double2* t[2] = {t0, t1};
+    for (int x = 0; x < 2; ++x) {
+        Zmm& q = first.p[nf++] = zmm(al, br, bl, e, false, ld, ZMM_N, gptr(b, s, x), !is64(b), ld, ZMM_N, t[x], ld);
+        q.scale_a = seen;
+    }
+    Zmm& q = second.p[ns++] = zmm(ar, br, al, gptr(a, s, 0), !is64(a), ld, ZMM_C, t0, false, ld, ZMM_N, en, ld);
+    q.a[1] = gptr(a, s, 1);
+    q.b[1] = t1;
+    q.segments = 2;
+    q.rowscale = lam_ptr(a, s);
+    q.colscale = lam_ptr(b, s);
+    q.largest = next;
+}
+
+// The same for the right environment `f` of site s (bra index down the rows) and that of site s - 1.
+void right_step(ptebd_state* a, ptebd_state* b, const std::vector<int32_t>& ca, const std::vector<int32_t>& cb, int s,
+                const double2* f, double2* fn, double2* t0, double2* t1, const unsigned long long* seen,
+                unsigned long long* next, ZmmBatch& first, int& nf, ZmmBatch& second, int& ns) {
+    const int ld = a->L.chip, al = ca[s], ar = ca[s + 1], bl = cb[s], br = cb[s + 1];
+    double2* t[2] = {t0, t1};
+    for (int x = 0; x < 2; ++x) {
+        Zmm& q = first.p[nf++] = zmm(al, br, ar, gptr(a, s, x), !is64(a), ld, ZMM_J, f, false, ld, ZMM_N, t[x], ld);
+        q.scale_b = seen;
+    }
+    Zmm& q = second.p[ns++] = zmm(al, bl, br, t0, false, ld, ZMM_N, gptr(b, s, 0), !is64(b), ld, ZMM_T, fn, ld);
+    q.a[1] = t1;
+    q.b[1] = gptr(b, s, 1);
+    q.segments = 2;
+    q.rowscale = lam_ptr(a, s - 1);
+    q.colscale = lam_ptr(b, s - 1);
+    q.largest = next;
+}
+
+// The overlaps of <a| and |b> with the physical indices of `width` sites (1 or 2) from
+// `site` left open: g[(bra), (ket)], 2^width values each, times 2^exponent.
+int open_overlaps(ptebd_state* a, ptebd_state* b, int site, int width, std::vector<double2>& g, double* exponent) {
+    Chain ch = chain_of(a);
+    cudaStream_t st = a->stream;
     int rc;
     std::vector<int32_t> ca = host_chi(a, &rc);
     if (rc) return rc;
-    std::vector<int32_t> cb = host_chi(b, &rc);
+    std::vector<int32_t> cb = a == b ? ca : host_chi(b, &rc);
     if (rc) return rc;
-    const int N = a->L.n_sites, lda_a = a->L.chip, lda_b = b->L.chip, ldc = own->L.chip;
-    double2* E = ch.mat[0];
-    double2* En = ch.mat[1];
-    CUDA_TRY(own, cudaMemsetAsync(ch.logacc, 0, sizeof(double), own->stream));
-    CUDA_TRY(own, launch_fill_identity(E, 1, 1, ldc, own->stream));
-    auto opc = [&](int r, int c, int dim) { return make_double2(op[2 * (r * dim + c)], op[2 * (r * dim + c) + 1]); };
-    int s = 0;
-    while (s < N) {
-        const int al = ca[s], ar = ca[s + 1], bl = cb[s], br = cb[s + 1];
-        const double* lamA = lam_ptr(a, s);
-        const double* lamB = lam_ptr(b, s);
-        if (s == site1) {
-            // T_x = sum_y O[x,y] E M_b[y];  E' = sum_x M_a[x]^dag T_x
-            for (int x = 0; x < 2; ++x)
-                for (int y = 0; y < 2; ++y)
-                    if ((rc = gemm(own, al, br, bl, opc(x, y, 2), E, true, ldc, 0, gptr(b, s, y), is64(b), lda_b, lamB,
-                                   y == 0 ? ZERO : ONE, ch.mat[2 + x], ldc, nullptr)))
-                        return rc;
-            for (int x = 0; x < 2; ++x)
-                if ((rc = gemm(own, ar, br, al, ONE, gptr(a, s, x), is64(a), lda_a, 1, ch.mat[2 + x], true, ldc,
-                               nullptr, x == 0 ? ZERO : ONE, En, ldc, lamA)))
-                    return rc;
-            s += 1;
-        } else if (s == site2) {
-            const int bm = cb[s + 2], am = ca[s + 2];
-            const double* lamB2 = lam_ptr(b, s + 1);
-            const double* lamA2 = lam_ptr(a, s + 1);
-            // R_y = E M_b,s[y]  (al x br)
-            for (int y = 0; y < 2; ++y)
-                if ((rc = gemm(own, al, br, bl, ONE, E, true, ldc, 0, gptr(b, s, y), is64(b), lda_b, lamB, ZERO,
-                               ch.mat[2 + y], ldc, nullptr)))
-                    return rc;
-            // X_xz = sum_{y,w} O[(x z), (y w)] R_y M_b,s+1[w]   (al x bm)
-            for (int x = 0; x < 2; ++x)
-                for (int z = 0; z < 2; ++z) {
-                    double2* X = ch.mat[4 + 2 * x + z];
-                    bool first = true;
-                    for (int y = 0; y < 2; ++y)
-                        for (int w = 0; w < 2; ++w) {
-                            if ((rc = gemm(own, al, bm, br, opc(2 * x + z, 2 * y + w, 4), ch.mat[2 + y], true, ldc, 0,
-                                           gptr(b, s + 1, w), is64(b), lda_b, lamB2, first ? ZERO : ONE, X, ldc,
-                                           nullptr)))
-                                return rc;
-                            first = false;
-                        }
-                }
-            // E' = sum_{x,z} M_a,s+1[z]^dag (M_a,s[x]^dag X_xz)
-            bool firstE = true;
-            for (int x = 0; x < 2; ++x)
-                for (int z = 0; z < 2; ++z) {
-                    double2* Y = ch.mat[2];
-                    if ((rc = gemm(own, ar, bm, al, ONE, gptr(a, s, x), is64(a), lda_a, 1, ch.mat[4 + 2 * x + z], true,
-                                   ldc, nullptr, ZERO, Y, ldc, lamA)))
-                        return rc;
-                    if ((rc = gemm(own, am, bm, ar, ONE, gptr(a, s + 1, z), is64(a), lda_a, 1, Y, true, ldc, nullptr,
-                                   firstE ? ZERO : ONE, En, ldc, lamA2)))
-                        return rc;
-                    firstE = false;
-                }
-            s += 2;
-        } else {
-            for (int x = 0; x < 2; ++x) {
-                if ((rc = gemm(own, al, br, bl, ONE, E, true, ldc, 0, gptr(b, s, x), is64(b), lda_b, lamB, ZERO,
-                               ch.mat[2], ldc, nullptr)))
-                    return rc;
-                if ((rc = gemm(own, ar, br, al, ONE, gptr(a, s, x), is64(a), lda_a, 1, ch.mat[2], true, ldc, nullptr,
-                               x == 0 ? ZERO : ONE, En, ldc, lamA)))
-                    return rc;
-            }
-            s += 1;
+    const int N = a->L.n_sites, ld = a->L.chip;
+    const int nl = site, nr = N - site - width;  // steps from each end
+    double2 *e = ch.mat[0], *en = ch.mat[1], *f = ch.mat[2], *fn = ch.mat[3];
+    unsigned long long *le = nullptr, *lf = nullptr, *free_l = ch.largest;
+    CUDA_TRY(a, launch_chain_start(e, f, ch.largest, N + 2, st));
+    for (int s = 0; s < std::max(nl, nr); ++s) {
+        ZmmBatch first, second;
+        int nf = 0, ns = 0;
+        unsigned long long *ne = le, *nx = lf;
+        if (s < nl) {
+            ne = free_l++;
+            left_step(a, b, ca, cb, s, e, en, ch.mat[4], ch.mat[5], le, ne, first, nf, second, ns);
         }
-        const int rows = ca[s], cols = cb[s];
-        CUDA_TRY(own, launch_scale_max(En, rows, cols, ldc, ch.logacc, own->stream));
-        std::swap(E, En);
+        if (s < nr) {
+            nx = free_l++;
+            right_step(a, b, ca, cb, N - 1 - s, f, fn, ch.mat[6], ch.mat[7], lf, nx, first, nf, second, ns);
+        }
+        CUDA_TRY(a, launch_zmm(first, nf, st));
+        CUDA_TRY(a, launch_zmm(second, ns, st));
+        if (s < nl) { std::swap(e, en); le = ne; }
+        if (s < nr) { std::swap(f, fn); lf = nx; }
     }
-    double2 e00;
-    double lg;
-    CUDA_TRY(own, cudaMemcpyAsync(&e00, E, sizeof e00, cudaMemcpyDeviceToHost, own->stream));
-    CUDA_TRY(own, cudaMemcpyAsync(&lg, ch.logacc, sizeof lg, cudaMemcpyDeviceToHost, own->stream));
-    CUDA_TRY(own, cudaStreamSynchronize(own->stream));
-    const double sc = std::exp(lg);
-    out[0] = e00.x * sc;
-    out[1] = e00.y * sc;
+    const int n_largest = (int)(free_l - ch.largest);
+    const size_t slice = (size_t)ld * ld;
+    ZmmBatch m{};
+    if (width == 1) {
+        // K_y = E Gamma_b[y], Q_y = K_y F^T, g = <Gamma_a[x], Q_y>
+        const int al = ca[site], ar = ca[site + 1], bl = cb[site], br = cb[site + 1];
+        for (int y = 0; y < 2; ++y) {
+            m.p[y] = zmm(al, br, bl, e, false, ld, ZMM_N, gptr(b, site, y), !is64(b), ld, ZMM_N, ch.mat[4 + y], ld);
+            m.p[y].scale_a = le;
+        }
+        CUDA_TRY(a, launch_zmm(m, 2, st));
+        for (int y = 0; y < 2; ++y) {
+            m.p[y] = zmm(al, ar, br, ch.mat[4 + y], false, ld, ZMM_N, f, false, ld, ZMM_T, ch.mat[6 + y], ld);
+            m.p[y].scale_b = lf;
+        }
+        CUDA_TRY(a, launch_zmm(m, 2, st));
+        CUDA_TRY(a, launch_overlaps(gptr(a, site, 0), !is64(a), slice, ld, 2, ch.mat[6], slice, ld, 2, al, ar, ch.out,
+                                    ch.largest, n_largest, ch.exponent, st));
+    } else {
+        // A_y = E Gamma_b[y] Lambda_b, B_w = Gamma_b'[w] F^T, C_yw = A_y B_w and
+        // D_xz = Gamma_a[x] Lambda_a Gamma_a'[z]; g = <D_xz, C_yw>
+        const int al = ca[site], am = ca[site + 1], ar = ca[site + 2];
+        const int bl = cb[site], bm = cb[site + 1], br = cb[site + 2];
+        for (int y = 0; y < 2; ++y) {
+            m.p[y] = zmm(al, bm, bl, e, false, ld, ZMM_N, gptr(b, site, y), !is64(b), ld, ZMM_N, ch.mat[4 + y], ld);
+            m.p[y].scale_a = le;
+            m.p[y].colscale = lam_ptr(b, site);
+            m.p[2 + y] = zmm(bm, ar, br, gptr(b, site + 1, y), !is64(b), ld, ZMM_N, f, false, ld, ZMM_T, ch.mat[6 + y], ld);
+            m.p[2 + y].scale_b = lf;
+        }
+        CUDA_TRY(a, launch_zmm(m, 4, st));
+        for (int x = 0; x < 2; ++x)
+            for (int z = 0; z < 2; ++z) {
+                m.p[2 * x + z] = zmm(al, ar, bm, ch.mat[4 + x], false, ld, ZMM_N, ch.mat[6 + z], false, ld, ZMM_N,
+                                     ch.mat[8 + 2 * x + z], ld);
+                Zmm& d = m.p[4 + 2 * x + z] = zmm(al, ar, am, gptr(a, site, x), !is64(a), ld, ZMM_N,
+                                                  gptr(a, site + 1, z), !is64(a), ld, ZMM_N, ch.mat[12 + 2 * x + z], ld);
+                d.kscale = lam_ptr(a, site);
+            }
+        CUDA_TRY(a, launch_zmm(m, 8, st));
+        CUDA_TRY(a, launch_overlaps(ch.mat[12], false, slice, ld, 4, ch.mat[8], slice, ld, 4, al, ar, ch.out, ch.largest,
+                                    n_largest, ch.exponent, st));
+    }
+    const int ng = width == 1 ? 4 : 16;
+    double2 host[17];  // the overlaps and, behind all sixteen, the exponent
+    CUDA_TRY(a, cudaMemcpyAsync(host, ch.out, sizeof host, cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(a, cudaStreamSynchronize(st));
+    g.assign(host, host + ng);
+    *exponent = host[16].x;
     return PTEBD_OK;
 }
 
-// Left environments E_0..E_{N-1} of `st` (E_0 = (1); E_{s+1} = sum_x M_s[x]^dag E_s M_s[x]),
-// each rescaled by its largest modulus, written to env[s] (chip x chip complex128).
-int left_envs(ptebd_state* st, const std::vector<int32_t>& chi, double2* env, double* logacc) {
-    const int N = st->L.n_sites, ld = st->L.chip;
-    const size_t slice = (size_t)ld * ld;
-    Chain ch = chain_of(st);
-    CUDA_TRY(st, launch_fill_identity(env, 1, 1, ld, st->stream));
-    int rc;
-    for (int s = 0; s + 1 < N; ++s) {
-        const int al = chi[s], ar = chi[s + 1];
-        double2* E = env + (size_t)s * slice;
-        double2* En = env + (size_t)(s + 1) * slice;
-        const double* lam = lam_ptr(st, s);
-        for (int x = 0; x < 2; ++x) {
-            if ((rc = gemm(st, al, ar, al, ONE, E, true, ld, 0, gptr(st, s, x), is64(st), ld, lam, ZERO, ch.mat[2],
-                           ld, nullptr)))
-                return rc;
-            if ((rc = gemm(st, ar, ar, al, ONE, gptr(st, s, x), is64(st), ld, 1, ch.mat[2], true, ld, nullptr,
-                           x == 0 ? ZERO : ONE, En, ld, lam)))
-                return rc;
+// <a|b>, contracted from both ends to the middle.
+int contract(ptebd_state* a, ptebd_state* b, double out[2]) {
+    std::vector<double2> g;
+    double ex;
+    int rc = open_overlaps(a, b, a->L.n_sites / 2, 1, g, &ex);
+    if (rc) return rc;
+    const int e = (int)ex;
+    out[0] = std::ldexp(g[0].x + g[3].x, e);
+    out[1] = std::ldexp(g[0].y + g[3].y, e);
+    return PTEBD_OK;
+}
+
+// <st| op |st> / <st|st>, op (row-major complex, 2^width squared) on `width` sites from `site`.
+int expectation(ptebd_state* st, int site, int width, const double* op, double out[2]) {
+    std::vector<double2> g;
+    double ex;
+    int rc = open_overlaps(st, st, site, width, g, &ex);
+    if (rc) return rc;
+    const int d = 1 << width;
+    double nx = 0.0, ny = 0.0, den = 0.0;
+    for (int r = 0; r < d; ++r) {
+        den += g[r * d + r].x;
+        for (int c = 0; c < d; ++c) {
+            const double ox = op[2 * (r * d + c)], oy = op[2 * (r * d + c) + 1];
+            const double2 v = g[r * d + c];
+            nx += ox * v.x - oy * v.y;
+            ny += ox * v.y + oy * v.x;
         }
-        CUDA_TRY(st, launch_scale_max(En, ar, ar, ld, logacc, st->stream));
+    }
+    out[0] = nx / den;
+    out[1] = ny / den;
+    return PTEBD_OK;
+}
+
+// Left environments E_0..E_{N-1} of `st` (E_0 = (1); E_{s+1} = sum_x M_s[x]^dag E_s M_s[x]), each
+// up to a power of two, written to env[s] (chip x chip complex128).
+int left_envs(ptebd_state* st, const std::vector<int32_t>& chi, double2* env) {
+    const int N = st->L.n_sites;
+    const size_t slice = (size_t)st->L.chip * st->L.chip;
+    Chain ch = chain_of(st);
+    CUDA_TRY(st, launch_chain_start(env, nullptr, ch.largest, N + 2, st->stream));
+    for (int s = 0; s + 1 < N; ++s) {
+        ZmmBatch first, second;
+        int nf = 0, ns = 0;
+        left_step(st, st, chi, chi, s, env + s * slice, env + (s + 1) * slice, ch.mat[4], ch.mat[5],
+                  s ? ch.largest + s - 1 : nullptr, ch.largest + s, first, nf, second, ns);
+        CUDA_TRY(st, launch_zmm(first, nf, st->stream));
+        CUDA_TRY(st, launch_zmm(second, ns, st->stream));
     }
     return PTEBD_OK;
 }
@@ -1201,7 +1241,7 @@ int ptebd_norm(ptebd_state* st, double* out) {
     int rc = sync_and_check(st);
     if (rc) return rc;
     double v[2];
-    rc = contract(st, st, -1, -1, nullptr, v);
+    rc = contract(st, st, v);
     if (rc) return rc;
     *out = std::sqrt(std::max(v[0], 0.0));
     return PTEBD_OK;
@@ -1214,7 +1254,7 @@ int ptebd_overlap(ptebd_state* a, ptebd_state* b, double out[2]) {
     int rc = sync_and_check(a);
     if (rc) return rc;
     if ((rc = sync_and_check(b))) return rc;
-    return contract(a, b, -1, -1, nullptr, out);
+    return contract(a, b, out);
 }
 
 int ptebd_expect(ptebd_state* st, int32_t site, const double* op, double out[2]) {
@@ -1222,12 +1262,7 @@ int ptebd_expect(ptebd_state* st, int32_t site, const double* op, double out[2])
     if (site < 0 || site >= st->L.n_sites) return set_err(st, PTEBD_ERR_INVALID, "site out of range");
     int rc = sync_and_check(st);
     if (rc) return rc;
-    double num[2], den[2];
-    if ((rc = contract(st, st, site, -1, op, num))) return rc;
-    if ((rc = contract(st, st, -1, -1, nullptr, den))) return rc;
-    out[0] = num[0] / den[0];
-    out[1] = num[1] / den[0];
-    return PTEBD_OK;
+    return expectation(st, site, 1, op, out);
 }
 
 int ptebd_expect2(ptebd_state* st, int32_t site, const double* op, double out[2]) {
@@ -1235,12 +1270,7 @@ int ptebd_expect2(ptebd_state* st, int32_t site, const double* op, double out[2]
     if (site < 0 || site >= st->L.n_sites - 1) return set_err(st, PTEBD_ERR_INVALID, "site out of range");
     int rc = sync_and_check(st);
     if (rc) return rc;
-    double num[2], den[2];
-    if ((rc = contract(st, st, -1, site, op, num))) return rc;
-    if ((rc = contract(st, st, -1, -1, nullptr, den))) return rc;
-    out[0] = num[0] / den[0];
-    out[1] = num[1] / den[0];
-    return PTEBD_OK;
+    return expectation(st, site, 2, op, out);
 }
 
 int ptebd_get_chi(ptebd_state* st, int32_t* chi_out) {
@@ -1529,18 +1559,44 @@ int ptebd_canonicalize(ptebd_state* st) {
 }
 
 namespace {
-size_t sample_ws_bytes(int n_sites, int chip, int n_samples) {
-    const int batch = std::max(1, std::min(n_samples, 1024));
-    // N environments, two vector buffers, uniforms and bits of one batch, one log accumulator
-    return align256((size_t)n_sites * chip * chip * sizeof(double2)) +
-           2 * align256((size_t)batch * chip * sizeof(double2)) + align256((size_t)batch * n_sites * sizeof(double)) +
-           align256((size_t)batch * n_sites * sizeof(int32_t)) + 256;
+// Workspace of the sampling: N environments, then for a batch of samples the vectors
+// v, t_0, t_1, u_0, u_1, the uniforms and the bits.
+struct SampleWs {
+    double2 *env, *v, *t, *u;
+    double* uniforms;
+    int32_t* bits;
+    size_t bytes;
+};
+// `vectors`: with t and u (they may also lie in the state's scratch)
+SampleWs sample_ws(char* w, int n_sites, int chip, int batch, bool vectors) {
+    SampleWs r{};
+    const size_t vec = align256((size_t)batch * chip * sizeof(double2));
+    size_t o = 0;
+    auto take = [&](size_t bytes) { char* p = w + o; o += align256(bytes); return p; };
+    r.env = reinterpret_cast<double2*>(take((size_t)n_sites * chip * chip * sizeof(double2)));
+    r.v = reinterpret_cast<double2*>(take(vec));
+    r.t = vectors ? reinterpret_cast<double2*>(take(2 * vec)) : nullptr;
+    r.u = vectors ? reinterpret_cast<double2*>(take(2 * vec)) : nullptr;
+    r.uniforms = reinterpret_cast<double*>(take((size_t)batch * n_sites * sizeof(double)));
+    r.bits = reinterpret_cast<int32_t*>(take((size_t)batch * n_sites * sizeof(int32_t)));
+    r.bytes = o;
+    return r;
+}
+int sample_batch(int n_samples) { return std::max(1, std::min(n_samples, 1024)); }
+// What a call needs at least: the environments, and for a whole batch two vectors,
+// the uniforms and the bits (smaller batches then make room for t and u).
+size_t sample_min_bytes(int n_sites, int chip, int n_samples) {
+    const size_t b = (size_t)sample_batch(n_samples);
+    return align256((size_t)n_sites * chip * chip * sizeof(double2)) + 2 * align256(b * chip * sizeof(double2)) +
+           align256(b * n_sites * sizeof(double)) + align256(b * n_sites * sizeof(int32_t)) + 256;
 }
 }  // namespace
 
 int ptebd_sample_workspace_bytes(const ptebd_state* st, int32_t n_samples, size_t* bytes) {
     if (!st || n_samples < 0 || !bytes) return PTEBD_ERR_INVALID;
-    *bytes = sample_ws_bytes(st->L.n_sites, st->L.chip, n_samples);
+    const int N = st->L.n_sites, chip = st->L.chip;
+    *bytes = std::max(sample_min_bytes(N, chip, n_samples),
+                      sample_ws(nullptr, N, chip, sample_batch(n_samples), true).bytes);
     return PTEBD_OK;
 }
 
@@ -1555,43 +1611,45 @@ int ptebd_sample(ptebd_state* st, int32_t n_samples, const double* uniforms, int
     if (rc) return rc;
     std::vector<int32_t> chi = host_chi(st, &rc);
     if (rc) return rc;
-    const int N = st->L.n_sites;
-    const size_t chip = (size_t)st->L.chip, slice = chip * chip;
-    const int batch = std::min(n_samples, 1024);
-    const size_t vec_bytes = (size_t)batch * chip * sizeof(double2);
-    const size_t need = sample_ws_bytes(N, (int)chip, n_samples);
+    const int N = st->L.n_sites, chip = st->L.chip;
+    const size_t slice = (size_t)chip * chip, need = sample_min_bytes(N, chip, n_samples);
     char* w = workspace ? static_cast<char*>(workspace) : st->ws;
     const size_t have = workspace ? workspace_bytes : st->ws_bytes;
     if (need > have)
         return set_err(st, PTEBD_ERR_MEMORY, "sampling needs %zu workspace bytes, %zu given", need, have);
-    double2* env = reinterpret_cast<double2*>(w); w += align256((size_t)N * slice * sizeof(double2));
-    double2* va = reinterpret_cast<double2*>(w); w += align256(vec_bytes);
-    double2* vb = reinterpret_cast<double2*>(w); w += align256(vec_bytes);
-    double* du = reinterpret_cast<double*>(w); w += align256((size_t)batch * N * sizeof(double));
-    int32_t* db = reinterpret_cast<int32_t*>(w); w += align256((size_t)batch * N * sizeof(int32_t));
-    double* logacc = reinterpret_cast<double*>(w);
-    CUDA_TRY(st, cudaMemsetAsync(logacc, 0, sizeof(double), st->stream));
-    if ((rc = left_envs(st, chi, env, logacc))) return rc;
+    // as many samples at once as the workspace holds with their t and u; a workspace that
+    // holds only a few runs up to chip samples with t and u in the state's scratch
+    int batch = sample_batch(n_samples);
+    while (batch > 0 && sample_ws(w, N, chip, batch, true).bytes > have) batch = batch > 64 ? batch - 64 : batch - 1;
+    const bool own = batch < std::min(sample_batch(n_samples), chip);
+    if (own) batch = std::min(sample_batch(n_samples), chip);
+    const SampleWs ws = sample_ws(w, N, chip, batch, !own);
+    Chain ch = chain_of(st);
+    double2* t = own ? ch.mat[8] : ws.t;   // (after the environments, which use mat[4] and mat[5])
+    double2* u = own ? ch.mat[10] : ws.u;
+    const size_t step = own ? slice : align256((size_t)batch * chip * sizeof(double2)) / sizeof(double2);
+    if ((rc = left_envs(st, chi, ws.env))) return rc;
     for (int k0 = 0; k0 < n_samples; k0 += batch) {
         const int nb = std::min(batch, n_samples - k0);
-        CUDA_TRY(st, cudaMemcpyAsync(du, uniforms + (size_t)k0 * N, (size_t)nb * N * sizeof(double),
+        CUDA_TRY(st, cudaMemcpyAsync(ws.uniforms, uniforms + (size_t)k0 * N, (size_t)nb * N * sizeof(double),
                                      cudaMemcpyHostToDevice, st->stream));
-        const double2* vin = nullptr;  // the right boundary: v = (1)
-        double2* vout = va;
+        CUDA_TRY(st, launch_sample_start(ws.v, chip, nb, st->stream));
         for (int s = N - 1; s >= 0; --s) {
             const int chil = chi[s], chir = chi[s + 1];
-            cudaError_t e;
-            if (is64(st))
-                e = launch_sample_site<double2>(gamma_ptr<double2>(st, s, 0), lam_ptr(st, s), chil, chir, (int)chip,
-                                                env + (size_t)s * slice, vin, vout, du, s, N, db, nb, st->stream);
-            else
-                e = launch_sample_site<float2>(gamma_ptr<float2>(st, s, 0), lam_ptr(st, s), chil, chir, (int)chip,
-                                               env + (size_t)s * slice, vin, vout, du, s, N, db, nb, st->stream);
-            if (e != cudaSuccess) return set_err(st, PTEBD_ERR_CUDA, "sampling launch failed: %s", cudaGetErrorString(e));
-            vin = vout;
-            vout = (vout == va) ? vb : va;
+            ZmmBatch m;
+            for (int x = 0; x < 2; ++x) {
+                m.p[x] = zmm(chil, nb, chir, gptr(st, s, x), !is64(st), chip, ZMM_N, ws.v, false, chip, ZMM_N,
+                             t + x * step, chip);
+                m.p[x].kscale = lam_ptr(st, s);
+            }
+            CUDA_TRY(st, launch_zmm(m, 2, st->stream));
+            for (int x = 0; x < 2; ++x)
+                m.p[x] = zmm(chil, nb, chil, ws.env + (size_t)s * slice, false, chip, ZMM_N, t + x * step, false, chip,
+                             ZMM_N, u + x * step, chip);
+            CUDA_TRY(st, launch_zmm(m, 2, st->stream));
+            CUDA_TRY(st, launch_sample_pick(t, u, step, chil, chip, ws.v, ws.uniforms, s, N, ws.bits, nb, st->stream));
         }
-        CUDA_TRY(st, cudaMemcpyAsync(bits + (size_t)k0 * N, db, (size_t)nb * N * sizeof(int32_t),
+        CUDA_TRY(st, cudaMemcpyAsync(bits + (size_t)k0 * N, ws.bits, (size_t)nb * N * sizeof(int32_t),
                                      cudaMemcpyDeviceToHost, st->stream));
         CUDA_TRY(st, cudaStreamSynchronize(st->stream));
     }

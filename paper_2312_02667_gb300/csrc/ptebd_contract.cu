@@ -1,12 +1,28 @@
-// Full contractions of an MPS (norm, overlap, expectation values) by
-// left-to-right transfer matrices E <- sum_s M_a[s]^dag E M_b[s], M = Gamma Lambda
-// (the MPS decomposition of Sec. II A-B of arXiv:2312.02667), with every
-// product accumulated in FP64.  Building blocks:
-//   k_zgemm       : C = alpha * rowscale o (op(A) * (B o colscale)) + beta * C,
-//                   column-major, complex64/complex128 inputs, complex128 output;
-//   k_scale_max   : divide E by its largest modulus and add the log to an
-//                   accumulator, so that long chains neither under- nor overflow;
-//   k_fill_identity.
+// Full contractions of an MPS (norm, overlap, expectation values, left
+// environments of the sampling) by transfer matrices, every product accumulated
+// in FP64 (the MPS decomposition of Sec. II A-B of arXiv:2312.02667).
+//
+// A contraction runs from both ends of the chain at once: the left environment
+// E' = sum_x Gamma_a[x]^dag E Gamma_b[x] and the right one
+// F' = sum_x conj(Gamma_a[x]) F Gamma_b[x]^T, each with the Lambda of its outer
+// bond on both sides, take a step in the same two launches (T_x = E Gamma_b[x],
+// conj(Gamma_a[x]) F; then the sums over x).  They meet at the site of the operator
+// (or in the middle), where the four or sixteen overlaps of Gamma_a[x] with
+// E Gamma_b[y] F^T are taken: an expectation value is a sum of those with the
+// operator's entries over their trace, so numerator and denominator share
+// everything.
+//
+//   k_zmm     : a batch of up to four complex products, k in one or two segments,
+//               rows and columns scaled, with the largest modulus of the result
+//               gathered so that the next step can take a power of two out;
+//   k_overlaps: sums of conj(P) Q;
+//   k_sample_pick.
+//
+// What bounds it: the FP64 pipe (2 fused multiply-adds per SM and cycle: a 64 x 64 x
+// 64 complex product is 3.5 us of the whole chip) and, at small bond dimensions, the
+// latency of a launch.  Hence 8 x 8 output tiles of 64 threads: chi = 64 gives 128
+// tiles a side (32 x 32 tiles of 256 threads kept 4 of 152 SMs busy at 65 us a
+// product), and two launches a step for both sides instead of five for one.
 #include <cmath>
 
 #include "ptebd_internal.h"
@@ -15,236 +31,241 @@ namespace ptebd {
 
 namespace {
 
-__device__ __forceinline__ double2 ld2(const float2 v) { return make_double2(v.x, v.y); }
-__device__ __forceinline__ double2 ld2(const double2 v) { return v; }
+// entry `i` of a complex64 or complex128 matrix
+__device__ __forceinline__ double2 entry(const void* p, size_t i, bool f32) {
+    if (f32) {
+        const float2 v = static_cast<const float2*>(p)[i];
+        return make_double2(v.x, v.y);
+    }
+    return static_cast<const double2*>(p)[i];
+}
 
-// grid (ceil(m/32), ceil(n/32)), 256 threads, 2x2 outputs per thread.
-template <typename TA, typename TB>
-__global__ void __launch_bounds__(256) k_zgemm(int m, int n, int k, double2 alpha, const TA* __restrict__ A,
-                                               int lda, int opA, const TB* __restrict__ B, int ldb,
-                                               const double* __restrict__ colscale, double2 beta,
-                                               double2* __restrict__ Cm, int ldc, const double* __restrict__ rowscale) {
-    __shared__ double2 as[16][33];  // [kk][i]
-    __shared__ double2 bs[16][33];  // [kk][j]
-    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    double2 acc[2][2];
+// 2^-e of the largest modulus gathered in *bits (1 when there is none, or it is not finite)
+__device__ __forceinline__ double unit_scale(const unsigned long long* bits) {
+    if (!bits) return 1.0;
+    const int e = (int)(*bits >> 52) & 0x7ff;
+    if (e == 0 || e >= 2046) return 1.0;
+    return __longlong_as_double((long long)(2046 - e) << 52);
+}
+
+constexpr int kTile = 8, kChunk = 32, kThreads = 64;
+
+// grid (ceil(max m / 8), ceil(max n / 8), problems), 64 threads, one output each.
+// The chunk of k after the one being multiplied is already on its way from memory.
+__global__ void __launch_bounds__(kThreads) k_zmm(ZmmBatch batch) {
+    const Zmm& q = batch.p[blockIdx.z];
+    const int i0 = blockIdx.x * kTile, j0 = blockIdx.y * kTile;
+    if (i0 >= q.m || j0 >= q.n) return;
+    __shared__ double2 as[kChunk][kTile + 1], bs[kChunk][kTile + 1];
+    const int t = threadIdx.x, ti = t & 7, tj = t >> 3;
+    const int per = (q.k + kChunk - 1) / kChunk, chunks = per * q.segments;
+    double2 ra[4], rb[4];
+    // element e of a chunk: the index that is contiguous in memory runs fastest
+    auto fetch = [&](int c) {
+        const int seg = c >= per ? 1 : 0, k0 = (c - seg * per) * kChunk;
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) acc[i][q] = make_double2(0.0, 0.0);
-    for (int k0 = 0; k0 < k; k0 += 16) {
-        for (int e = threadIdx.x; e < 512; e += 256) {
+        for (int u = 0; u < 4; ++u) {
+            const int e = t + u * kThreads;
             int kk, ii;
-            if (opA) { kk = e & 15; ii = e >> 4; } else { ii = e & 31; kk = e >> 5; }
-            const int gi = i0 + ii, gk = k0 + kk;
+            if (q.op_a == ZMM_C) { kk = e & 31; ii = e >> 5; } else { ii = e & 7; kk = e >> 3; }
+            const int k = k0 + kk, i = i0 + ii;
             double2 v = make_double2(0.0, 0.0);
-            if (gi < m && gk < k) {
-                if (opA) { v = ld2(A[(size_t)gi * lda + gk]); v.y = -v.y; }
-                else v = ld2(A[(size_t)gk * lda + gi]);
+            if (k < q.k && i < q.m) {
+                const size_t at = q.op_a == ZMM_C ? (size_t)i * q.lda + k : (size_t)k * q.lda + i;
+                v = entry(q.a[seg], at, q.a32);
+                if (q.op_a != ZMM_N) v.y = -v.y;
+                if (q.kscale) { v.x *= q.kscale[k]; v.y *= q.kscale[k]; }
             }
-            as[kk][ii] = v;
-        }
-        for (int e = threadIdx.x; e < 512; e += 256) {
-            const int kk = e & 15, jj = e >> 4;
-            const int gj = j0 + jj, gk = k0 + kk;
-            double2 v = make_double2(0.0, 0.0);
-            if (gj < n && gk < k) {
-                v = ld2(B[(size_t)gj * ldb + gk]);
-                if (colscale) { v.x *= colscale[gj]; v.y *= colscale[gj]; }
+            ra[u] = v;
+            int kb, jj;
+            if (q.op_b == ZMM_T) { jj = e & 7; kb = e >> 3; } else { kb = e & 31; jj = e >> 5; }
+            const int k2 = k0 + kb, j = j0 + jj;
+            double2 w = make_double2(0.0, 0.0);
+            if (k2 < q.k && j < q.n) {
+                const size_t at = q.op_b == ZMM_T ? (size_t)k2 * q.ldb + j : (size_t)j * q.ldb + k2;
+                w = entry(q.b[seg], at, q.b32);
             }
-            bs[kk][jj] = v;
+            rb[u] = w;
         }
+    };
+    auto put = [&]() {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int e = t + u * kThreads;
+            if (q.op_a == ZMM_C) as[e & 31][e >> 5] = ra[u]; else as[e >> 3][e & 7] = ra[u];
+            if (q.op_b == ZMM_T) bs[e >> 3][e & 7] = rb[u]; else bs[e & 31][e >> 5] = rb[u];
+        }
+    };
+    double2 acc = make_double2(0.0, 0.0);
+    fetch(0);
+    for (int c = 0; c < chunks; ++c) {
+        put();
         __syncthreads();
-#pragma unroll 4
-        for (int kk = 0; kk < 16; ++kk) {
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const double2 x = as[kk][tx + 16 * i];
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const double2 y = bs[kk][ty + 16 * q];
-                    acc[i][q].x = fma(x.x, y.x, acc[i][q].x); acc[i][q].x = fma(-x.y, y.y, acc[i][q].x);
-                    acc[i][q].y = fma(x.x, y.y, acc[i][q].y); acc[i][q].y = fma(x.y, y.x, acc[i][q].y);
-                }
+        if (c + 1 < chunks) fetch(c + 1);
+        const int seg = c >= per ? 1 : 0, depth = min(kChunk, q.k - (c - seg * per) * kChunk);
+        if (depth == kChunk) {
+#pragma unroll 8
+            for (int kk = 0; kk < kChunk; ++kk) {
+                const double2 x = as[kk][ti], y = bs[kk][tj];
+                acc.x = fma(x.x, y.x, acc.x); acc.y = fma(x.x, y.y, acc.y);
+                acc.x = fma(-x.y, y.y, acc.x); acc.y = fma(x.y, y.x, acc.y);
+            }
+        } else {
+            for (int kk = 0; kk < depth; ++kk) {
+                const double2 x = as[kk][ti], y = bs[kk][tj];
+                acc.x = fma(x.x, y.x, acc.x); acc.y = fma(x.x, y.y, acc.y);
+                acc.x = fma(-x.y, y.y, acc.x); acc.y = fma(x.y, y.x, acc.y);
             }
         }
         __syncthreads();
     }
+    const int i = i0 + ti, j = j0 + tj;
+    double big = 0.0;
+    if (i < q.m && j < q.n) {
+        double f = unit_scale(q.scale_a) * unit_scale(q.scale_b);
+        if (q.rowscale) f *= q.rowscale[i];
+        if (q.colscale) f *= q.colscale[j];
+        acc.x *= f;
+        acc.y *= f;
+        static_cast<double2*>(q.c)[(size_t)j * q.ldc + i] = acc;
+        big = fmax(fabs(acc.x), fabs(acc.y));
+    }
+    if (q.largest) {
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int gi = i0 + tx + 16 * i, gj = j0 + ty + 16 * q;
-            if (gi >= m || gj >= n) continue;
-            double2 p = acc[i][q];
-            if (rowscale) { p.x *= rowscale[gi]; p.y *= rowscale[gi]; }
-            double2 r = make_double2(alpha.x * p.x - alpha.y * p.y, alpha.x * p.y + alpha.y * p.x);
-            double2* c = Cm + (size_t)gj * ldc + gi;
-            if (beta.x != 0.0 || beta.y != 0.0) {
-                const double2 o = *c;
-                r.x += beta.x * o.x - beta.y * o.y;
-                r.y += beta.x * o.y + beta.y * o.x;
-            }
-            *c = r;
-        }
+        for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+        if ((t & 31) == 0) atomicMax(q.largest, (unsigned long long)__double_as_longlong(big));
+    }
 }
 
-__global__ void __launch_bounds__(256) k_scale_max(double2* E, int rows, int cols, int ld, double* log_acc) {
-    __shared__ double red[256];
-    double mx = 0.0;
-    for (int e = threadIdx.x; e < rows * cols; e += 256) {
-        const double2 v = E[(size_t)(e / rows) * ld + (e % rows)];
-        mx = fmax(mx, fmax(fabs(v.x), fabs(v.y)));
+// (1) as the environments of both ends, and the exponents gathered along the chain cleared
+__global__ void __launch_bounds__(256) k_chain_start(double2* e, double2* f, unsigned long long* largest, int n) {
+    for (int i = threadIdx.x; i < n; i += 256) largest[i] = 0ull;
+    if (threadIdx.x == 0) {
+        if (e) e[0] = make_double2(1.0, 0.0);
+        if (f) f[0] = make_double2(1.0, 0.0);
     }
-    red[threadIdx.x] = mx;
+}
+
+// out[blockIdx.x]: sum over the m x n entries of conj(p) q, block x = pair (x / nq, x mod nq)
+// of the np matrices P (stride p_step entries) and the nq matrices Q; and, in one
+// block, out_exp = the power of two taken out along the chain.
+__global__ void __launch_bounds__(512) k_overlaps(const void* p, bool p32, size_t p_step, int ldp, const double2* q,
+                                                  size_t q_step, int ldq, int nq, int m, int n, double2* out,
+                                                  const unsigned long long* largest, int n_largest, double* out_exp) {
+    __shared__ double sx[512], sy[512];
+    const int t = threadIdx.x;
+    const size_t po = (size_t)(blockIdx.x / nq) * p_step, qo = (size_t)(blockIdx.x % nq) * q_step;
+    double x = 0.0, y = 0.0;
+    for (int e = t; e < m * n; e += 512) {
+        const int i = e % m, j = e / m;
+        const double2 u = entry(p, po + (size_t)j * ldp + i, p32), v = q[qo + (size_t)j * ldq + i];
+        x = fma(u.x, v.x, x); x = fma(u.y, v.y, x);
+        y = fma(u.x, v.y, y); y = fma(-u.y, v.x, y);
+    }
+    sx[t] = x;
+    sy[t] = y;
     __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + s]);
+    for (int s = 256; s > 0; s >>= 1) {
+        if (t < s) { sx[t] += sx[t + s]; sy[t] += sy[t + s]; }
         __syncthreads();
     }
-    const double m = red[0];
-    if (!(m > 0.0) || !isfinite(m)) return;  // a zero or broken chain stays as it is
-    const double inv = 1.0 / m;
-    for (int e = threadIdx.x; e < rows * cols; e += 256) {
-        double2* p = E + (size_t)(e / rows) * ld + (e % rows);
-        p->x *= inv; p->y *= inv;
+    if (t == 0) out[blockIdx.x] = make_double2(sx[0], sy[0]);
+    if (blockIdx.x == 0) {
+        __shared__ int se[512];
+        int sum = 0;
+        for (int i = t; i < n_largest; i += 512) {
+            const int e = (int)(largest[i] >> 52) & 0x7ff;
+            if (e != 0 && e < 2046) sum += e - 1023;
+        }
+        se[t] = sum;
+        __syncthreads();
+        for (int s = 256; s > 0; s >>= 1) {
+            if (t < s) se[t] += se[t + s];
+            __syncthreads();
+        }
+        if (t == 0) *out_exp = (double)se[0];
     }
-    if (threadIdx.x == 0) *log_acc += log(m);
 }
 
-__global__ void k_fill_identity(double2* E, int rows, int cols, int ld) {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < rows * cols; e += gridDim.x * blockDim.x) {
-        const int r = e % rows, c = e / rows;
-        E[(size_t)c * ld + r] = make_double2(r == c ? 1.0 : 0.0, 0.0);
-    }
-}
-
-// One sampling step at `site` (sites are drawn from the right end), one CTA per
-// sample: t_x = M_site[x] v (x = 0, 1; M = Gamma diag(Lambda_site)),
-// w_x = t_x^dag L t_x with L the left environment of the site, sigma = 0 when
-// u < w_0 / (w_0 + w_1); v <- t_sigma / |t_sigma|.
-// v_in: samples x chip (chir valid entries; nullptr = the unit vector (1) of the
-// right boundary), v_out: samples x chip (chil valid).
-template <typename TG>
-__global__ void __launch_bounds__(256) k_sample_site(const TG* __restrict__ gamma_s, const double* __restrict__ lam,
-                                                     int chil, int chir, int chip, const double2* __restrict__ L,
-                                                     const double2* __restrict__ v_in, double2* __restrict__ v_out,
+// One sampling decision at `site` for every sample (a warp each): w_x = t_x^dag u_x
+// with t_x = Gamma[x] Lambda v and u_x = L t_x, sigma = 0 when u < w_0 / (w_0 + w_1),
+// v <- t_sigma / |t_sigma|.  t, u: two matrices of chil x samples (ld chip), `step` apart.
+__global__ void __launch_bounds__(256) k_sample_pick(const double2* __restrict__ tm, const double2* __restrict__ um,
+                                                     size_t step, int chil, int chip, double2* __restrict__ v,
                                                      const double* __restrict__ uniforms, int site, int n_sites,
-                                                     int32_t* __restrict__ bits) {
-    __shared__ double2 vs[512];
-    __shared__ double2 ts[2][512];
-    __shared__ double red[3][256];
-    __shared__ int choice;
-    const int k = blockIdx.x, t = threadIdx.x;
-    const size_t slice = (size_t)chip * chip;
-    for (int b = t; b < chir; b += 256) {
-        double2 x = v_in ? v_in[(size_t)k * chip + b] : make_double2(b == 0 ? 1.0 : 0.0, 0.0);
-        x.x *= lam[b]; x.y *= lam[b];
-        vs[b] = x;
-    }
-    __syncthreads();
-    for (int a = t; a < chil; a += 256) {
-        double2 s0 = make_double2(0, 0), s1 = make_double2(0, 0);
-        for (int b = 0; b < chir; ++b) {
-            const double2 g0 = ld2(gamma_s[(size_t)b * chip + a]);
-            const double2 g1 = ld2(gamma_s[slice + (size_t)b * chip + a]);
-            const double2 x = vs[b];
-            s0.x += g0.x * x.x - g0.y * x.y; s0.y += g0.x * x.y + g0.y * x.x;
-            s1.x += g1.x * x.x - g1.y * x.y; s1.y += g1.x * x.y + g1.y * x.x;
+                                                     int32_t* __restrict__ bits, int samples) {
+    const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (k >= samples) return;
+    double w[2] = {0.0, 0.0}, nn[2] = {0.0, 0.0};
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const double2* tc = tm + x * step + (size_t)k * chip;
+        const double2* uc = um + x * step + (size_t)k * chip;
+        for (int a = lane; a < chil; a += 32) {
+            const double2 tv = tc[a], uv = uc[a];
+            w[x] += tv.x * uv.x + tv.y * uv.y;
+            nn[x] += tv.x * tv.x + tv.y * tv.y;
         }
-        ts[0][a] = s0;
-        ts[1][a] = s1;
-    }
-    __syncthreads();
-    // w_x = sum_a conj(t_x[a]) (L t_x)[a]; |t_x|^2 alongside
-    double w0 = 0.0, w1 = 0.0;
-    for (int a = t; a < chil; a += 256) {
-        double2 u0 = make_double2(0, 0), u1 = make_double2(0, 0);
-        for (int c = 0; c < chil; ++c) {
-            const double2 l = L[(size_t)c * chip + a];
-            const double2 x0 = ts[0][c], x1 = ts[1][c];
-            u0.x += l.x * x0.x - l.y * x0.y; u0.y += l.x * x0.y + l.y * x0.x;
-            u1.x += l.x * x1.x - l.y * x1.y; u1.y += l.x * x1.y + l.y * x1.x;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            w[x] += __shfl_xor_sync(0xffffffffu, w[x], o);
+            nn[x] += __shfl_xor_sync(0xffffffffu, nn[x], o);
         }
-        w0 += ts[0][a].x * u0.x + ts[0][a].y * u0.y;
-        w1 += ts[1][a].x * u1.x + ts[1][a].y * u1.y;
     }
-    red[0][t] = w0;
-    red[1][t] = w1;
-    __syncthreads();
-    for (int st = 128; st > 0; st >>= 1) {
-        if (t < st) { red[0][t] += red[0][t + st]; red[1][t] += red[1][t + st]; }
-        __syncthreads();
-    }
-    if (t == 0) {
-        const double p0 = red[0][0] / (red[0][0] + red[1][0]);
-        choice = uniforms[(size_t)k * n_sites + site] < p0 ? 0 : 1;
-        bits[(size_t)k * n_sites + site] = choice;
-    }
-    __syncthreads();
-    const int x = choice;
-    double nn = 0.0;
-    for (int a = t; a < chil; a += 256) nn += ts[x][a].x * ts[x][a].x + ts[x][a].y * ts[x][a].y;
-    red[2][t] = nn;
-    __syncthreads();
-    for (int st = 128; st > 0; st >>= 1) {
-        if (t < st) red[2][t] += red[2][t + st];
-        __syncthreads();
-    }
-    const double inv = red[2][0] > 0.0 ? 1.0 / sqrt(red[2][0]) : 0.0;
-    for (int a = t; a < chil; a += 256) {
-        double2 y = ts[x][a];
+    const double p0 = w[0] / (w[0] + w[1]);
+    const int x = uniforms[(size_t)k * n_sites + site] < p0 ? 0 : 1;
+    if (lane == 0) bits[(size_t)k * n_sites + site] = x;
+    const double n2 = x ? nn[1] : nn[0], inv = n2 > 0.0 ? 1.0 / sqrt(n2) : 0.0;
+    const double2* tc = tm + x * step + (size_t)k * chip;
+    for (int a = lane; a < chil; a += 32) {
+        double2 y = tc[a];
         y.x *= inv; y.y *= inv;
-        v_out[(size_t)k * chip + a] = y;
+        v[(size_t)k * chip + a] = y;
     }
+}
+
+// v_k = (1), the right boundary of every sample
+__global__ void k_sample_start(double2* v, int chip, int samples) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < samples) v[(size_t)k * chip] = make_double2(1.0, 0.0);
 }
 
 }  // namespace
 
-template <typename TG>
-cudaError_t launch_sample_site(const TG* gamma_s, const double* lam, int chil, int chir, int chip, const double2* L,
-                               const double2* v_in, double2* v_out, const double* uniforms, int site, int n_sites,
-                               int32_t* bits, int n_samples, cudaStream_t s) {
-    k_sample_site<TG><<<n_samples, 256, 0, s>>>(gamma_s, lam, chil, chir, chip, L, v_in, v_out, uniforms, site,
-                                                n_sites, bits);
-    return cudaGetLastError();
-}
-template cudaError_t launch_sample_site<float2>(const float2*, const double*, int, int, int, const double2*,
-                                                const double2*, double2*, const double*, int, int, int32_t*, int,
-                                                cudaStream_t);
-template cudaError_t launch_sample_site<double2>(const double2*, const double*, int, int, int, const double2*,
-                                                 const double2*, double2*, const double*, int, int, int32_t*, int,
-                                                 cudaStream_t);
-
-template <typename TA, typename TB>
-cudaError_t launch_zgemm(int m, int n, int k, double2 alpha, const TA* A, int lda, int opA, const TB* B, int ldb,
-                         const double* colscale_b, double2 beta, double2* Cm, int ldc, const double* rowscale_c,
-                         cudaStream_t s) {
-    if (m <= 0 || n <= 0) return cudaSuccess;
-    dim3 grid((m + 31) / 32, (n + 31) / 32);
-    k_zgemm<TA, TB><<<grid, 256, 0, s>>>(m, n, k, alpha, A, lda, opA, B, ldb, colscale_b, beta, Cm, ldc,
-                                         rowscale_c);
+cudaError_t launch_zmm(const ZmmBatch& b, int n, cudaStream_t s) {
+    int m = 0, c = 0;
+    for (int i = 0; i < n; ++i) {
+        m = b.p[i].m > m ? b.p[i].m : m;
+        c = b.p[i].n > c ? b.p[i].n : c;
+    }
+    if (m <= 0 || c <= 0) return cudaSuccess;
+    dim3 grid((m + kTile - 1) / kTile, (c + kTile - 1) / kTile, n);
+    k_zmm<<<grid, kThreads, 0, s>>>(b);
     return cudaGetLastError();
 }
 
-cudaError_t launch_scale_max(double2* E, int rows, int cols, int ld, double* log_acc, cudaStream_t s) {
-    k_scale_max<<<1, 256, 0, s>>>(E, rows, cols, ld, log_acc);
+cudaError_t launch_chain_start(double2* e, double2* f, unsigned long long* largest, int n, cudaStream_t s) {
+    k_chain_start<<<1, 256, 0, s>>>(e, f, largest, n);
     return cudaGetLastError();
 }
 
-cudaError_t launch_fill_identity(double2* E, int rows, int cols, int ld, cudaStream_t s) {
-    k_fill_identity<<<64, 256, 0, s>>>(E, rows, cols, ld);
+cudaError_t launch_overlaps(const void* p, bool p32, size_t p_step, int ldp, int np, const double2* q, size_t q_step,
+                            int ldq, int nq, int m, int n, double2* out, const unsigned long long* largest,
+                            int n_largest, double* out_exp, cudaStream_t s) {
+    k_overlaps<<<np * nq, 512, 0, s>>>(p, p32, p_step, ldp, q, q_step, ldq, nq, m, n, out, largest, n_largest, out_exp);
     return cudaGetLastError();
 }
 
-#define PTEBD_ZGEMM(TA, TB)                                                                                  \
-    template cudaError_t launch_zgemm<TA, TB>(int, int, int, double2, const TA*, int, int, const TB*, int, \
-                                              const double*, double2, double2*, int, const double*, cudaStream_t);
-PTEBD_ZGEMM(double2, double2)
-PTEBD_ZGEMM(double2, float2)
-PTEBD_ZGEMM(float2, double2)
-PTEBD_ZGEMM(float2, float2)
-#undef PTEBD_ZGEMM
+cudaError_t launch_sample_start(double2* v, int chip, int samples, cudaStream_t s) {
+    k_sample_start<<<(samples + 255) / 256, 256, 0, s>>>(v, chip, samples);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sample_pick(const double2* t, const double2* u, size_t step, int chil, int chip, double2* v,
+                               const double* uniforms, int site, int n_sites, int32_t* bits, int samples,
+                               cudaStream_t s) {
+    k_sample_pick<<<(samples + 7) / 8, 256, 0, s>>>(t, u, step, chil, chip, v, uniforms, site, n_sites, bits, samples);
+    return cudaGetLastError();
+}
 
 }  // namespace ptebd

@@ -54,7 +54,7 @@ enum : uint32_t {
 //   err    : latched error word
 //   gates  : ceil((N-1)/2) x 32 doubles, staging of host gates
 //   bonds  : 3 lists of ceil((N-1)/2) int32: even bonds, odd bonds, user list
-//   contraction scratch: 8 chip x chip complex128 matrices
+//   contraction scratch: kScratch chip x chip complex128 matrices, overlaps and exponents
 // Workspace (per slot = one bond of a chunk):
 //   w, w0, w1 : ldw x ldw complex each (ldw = 2 chip); w is rotated by the SVD,
 //            w0 keeps theta' (or its adjoint) for the second factor, w1 holds
@@ -123,6 +123,7 @@ enum { D_CL = 0, D_CM = 1, D_CR = 2, D_TALL = 3, D_BOND = 4, D_K = 5, D_ROWS = 6
        D_REFINE = 8, D_COND = 9 };
 constexpr int kDims = 16;
 constexpr int kWork = 16;  // work counters
+constexpr int kScratch = 16;  // chip x chip complex128 matrices of the contractions
 
 // ------------------------------------------------------------ launchers --
 // G: the complex type of the Gamma store (cx_t<R> except in the FP64 resolution)
@@ -152,19 +153,30 @@ constexpr int kMaxChunks = 16;
 template <typename R> cudaError_t jacobi_prepare();   // raises the dynamic smem limit
 int jacobi_block_width(int precision, int requested);  // the NW a launch with a.nw = requested uses
 
-// Transfer-matrix contraction.  C = rowscale o (op(A) B) o colscale * alpha + beta C,
-// all column-major; A and B are complex of type TA/TB, C is complex128.
-// opA: 0 = N, 1 = conjugate transpose.
-template <typename TA, typename TB>
-cudaError_t launch_zgemm(int m, int n, int k, double2 alpha,
-                         const TA* A, int lda, int opA, const TB* B, int ldb,
-                         const double* colscale_b, double2 beta, double2* Cm, int ldc,
-                         const double* rowscale_c, cudaStream_t s);
-template <typename TG>
-cudaError_t launch_sample_site(const TG* gamma_s, const double* lam, int chil, int chir, int chip, const double2* L,
-                               const double2* v_in, double2* v_out, const double* uniforms, int site, int n_sites,
-                               int32_t* bits, int n_samples, cudaStream_t s);
-cudaError_t launch_scale_max(double2* E, int rows, int cols, int ld, double* log_acc, cudaStream_t s);
-cudaError_t launch_fill_identity(double2* E, int rows, int cols, int ld, cudaStream_t s);
+// One product of a transfer-matrix contraction: C (m x n, complex128) =
+// rowscale o (sum over segments of op_a(A) op_b(B)) o colscale, all column-major,
+// times the powers of two that bring the largest moduli behind scale_a and scale_b
+// (of A's and B's last step) to [1, 2).  A and B are complex64 (a32, b32) or
+// complex128; kscale, if given, multiplies column k of op_a(A).
+enum { ZMM_N = 0, ZMM_C = 1, ZMM_J = 2, ZMM_T = 3 };  // as is, conjugate transpose, conjugate, transpose
+struct Zmm {
+    const void* a[2]; const void* b[2]; double2* c;
+    const double* kscale; const double* rowscale; const double* colscale;
+    const unsigned long long* scale_a; const unsigned long long* scale_b;
+    unsigned long long* largest;  // gathers the bits of the largest modulus of C (or null)
+    int m, n, k, segments, lda, ldb, ldc, op_a, op_b;  // op_a: N, C, J; op_b: N, T
+    bool a32, b32;
+};
+struct ZmmBatch { Zmm p[8]; };
+cudaError_t launch_zmm(const ZmmBatch& b, int n, cudaStream_t s);
+cudaError_t launch_chain_start(double2* e, double2* f, unsigned long long* largest, int n, cudaStream_t s);
+// out[p nq + q] = sum of conj(P_p) Q_q, p < np, q < nq; out_exp = sum of the exponents in largest[0..n_largest)
+cudaError_t launch_overlaps(const void* p, bool p32, size_t p_step, int ldp, int np, const double2* q, size_t q_step,
+                            int ldq, int nq, int m, int n, double2* out, const unsigned long long* largest,
+                            int n_largest, double* out_exp, cudaStream_t s);
+cudaError_t launch_sample_start(double2* v, int chip, int samples, cudaStream_t s);
+cudaError_t launch_sample_pick(const double2* t, const double2* u, size_t step, int chil, int chip, double2* v,
+                               const double* uniforms, int site, int n_sites, int32_t* bits, int samples,
+                               cudaStream_t s);
 
 }  // namespace ptebd
