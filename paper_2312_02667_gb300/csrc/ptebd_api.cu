@@ -46,6 +46,7 @@ struct ptebd_state {
     int chunk_streams = 0;  // requested number of chunks (0: chosen from N)
     int wait_test = 0;      // see ptebd_test_wait_timeout
     bool regauge64 = false; // PTEBD_MIXED: tSU stages run in FP64 (ptebd_set_regauge_precision)
+    int in_flight = 0;      // bonds of all the states of a batch whose layers run together (0: only this one)
     int jacobi_nw = 0;      // Jacobi block width (0: default; see ptebd_set_jacobi_width)
     int ptsu_shortcut = 1;  // leave out the identity half-step after a layer on bonds 0, 2, 4, ... (see run_layer)
     int tensor_cores = 1;   // complex64 theta' on the tensor cores (ptebd_set_tensor_cores)
@@ -364,7 +365,7 @@ LayerArgs<double> refine_args(ptebd_state* st, const LayerArgs<float>& c, int ba
     a.norms = c.norms; a.sig = c.sig; a.perm = c.perm; a.dims = c.dims;
     a.slot_eps = c.slot_eps; a.slot_lognu = c.slot_lognu; a.slot_sweeps = c.slot_sweeps;
     a.bonds = c.bonds; a.gates = c.gates;
-    a.count = c.count; a.chip = c.chip; a.ldw = c.ldw; a.n_sites = c.n_sites; a.chi_max = c.chi_max;
+    a.count = c.count; a.share = c.share; a.chip = c.chip; a.ldw = c.ldw; a.n_sites = c.n_sites; a.chi_max = c.chi_max;
     a.thr_rel = st->cfg.cutoff;
     a.resolve = 0.0;
     a.refine = 1;
@@ -494,6 +495,7 @@ int run_stage_serial(ptebd_state* st, const Stage& g) {
     for (int c0 = 0; c0 < g.nb; c0 += st->slots) {
         LayerArgs<R> a = stage_args<R>(st, g.gated);
         a.count = std::min(st->slots, g.nb - c0);
+        a.share = std::max(a.count, st->in_flight);
         a.bonds = g.d_list + c0;
         a.gates = g.gated ? g.d_gates + (size_t)c0 * 32 : nullptr;
         int rc = launch_chain<R>(st, a, 0, g.gated, st->stream, wrap);
@@ -549,6 +551,7 @@ int run_stages_chunked(ptebd_state* st, const std::vector<Stage>& stages, const 
             LayerArgs<R> a = stage_args<R>(st, g.gated);
             at_slots(a, L, c * p.cap);
             a.count = cnt[c];
+            a.share = std::max(g.nb, st->in_flight);
             a.bonds = g.d_list + off[c];
             a.gates = g.gated ? g.d_gates + (size_t)off[c] * 32 : nullptr;
             a.totals = part + 4 * c;
@@ -1514,8 +1517,12 @@ int ptebd_batch_apply_layer(ptebd_batch* b, const double* const* gates, const in
         cudaGraph_t graph = nullptr;
         if (cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) rc = PTEBD_ERR_CUDA;
         if (!rc && cudaEventRecord(b->ev[n], cap) != cudaSuccess) rc = PTEBD_ERR_CUDA;
+        int together = 0;
+        for (int i = 0; i < n; ++i)
+            if (key[i] >= 0) together += n_parity_bonds(b->states[i]->L.n_sites, key[i]);
         for (int i = 0; !rc && i < n; ++i) {
             ptebd_state* st = b->states[i];
+            st->in_flight = together;
             const cudaStream_t saved = st->stream;
             const bool timing = st->timing;
             st->timing = false;
@@ -1526,6 +1533,7 @@ int ptebd_batch_apply_layer(ptebd_batch* b, const double* const* gates, const in
             if (!rc && cudaStreamWaitEvent(cap, b->ev[i], 0) != cudaSuccess) rc = PTEBD_ERR_CUDA;
             st->stream = saved;
             st->timing = timing;
+            st->in_flight = 0;
         }
         const cudaError_t ee = cudaStreamEndCapture(cap, &graph);
         if (!rc && ee != cudaSuccess) rc = PTEBD_ERR_CUDA;

@@ -90,6 +90,7 @@ struct LayerArgs {
     double* slot_eps; double* slot_lognu; int32_t* slot_sweeps;
     const int32_t* bonds; const double* gates;  // gates == nullptr: tSU
     int count, chip, ldw, n_sites, chi_max;
+    int share;        // bonds of the whole stage or batch, over all launches that run together (0: count)
     double thr_rel;   // relative truncation threshold: the cutoff, or max(cutoff, resolve) when the
                       // complex64 spectrum decides a bond without the FP64 resolution
     double resolve;   // > thr_rel: bonds whose kept count depends on singular values <= resolve * sigma_1
@@ -105,7 +106,7 @@ struct LayerArgs {
     int wait_test;    // test of the bounded waits: one hand-off wait per CTA targets a count nothing
                       // reaches, with a short limit, so the CTA aborts and latches DERR_TIMEOUT
     int nw;           // Jacobi block width requested (complex64: 8 halves a CTA's warps and shared memory)
-    int tensor_cores; // complex64 on the tensor cores (tcgen05, 3xTF32) when chip >= 64: 1 theta' and
+    int tensor_cores; // complex64 on the tensor cores (tcgen05, 3xTF32) when chip >= 128: 1 theta' and
                       // the Gamma GEMM of gated stages, 2 the tSU steps as well
     int polish;       // complex64 Jacobi: one last sweep at the tighter threshold (see Eps::polish)
     int mode;         // 0: gated bond; 1: tSU through the rank-chi_b factorisation

@@ -49,6 +49,15 @@
 // in row-cyclic order: a tournament over all groups would keep every warp busy
 // but takes 13 to 16 sweeps where this order takes 10 or 11.
 //
+// With few matrices, each is spread over the CTAs of a cluster (kCluster): the
+// columns lie in the shared memory of all of them, the warps of all of them make
+// one row of I groups, and counters, norms and scales are read through distributed
+// shared memory.  The arithmetic and its order are the same, so the result does
+// not depend on how a matrix was spread.  10 complex128 256 x 256: 313 -> 71 ms
+// (8 CTAs each), 64 of 128 x 128: 41 -> 28 (2 each); complex64 37 of 200 x 200
+// 5.6 -> 3.6 (3 or 4 each).  Each launch takes the largest cluster at which all its
+// matrices still run at once (cluster_for).
+//
 // Every wait is bounded by a clock budget; one that runs out raises the CTA's
 // abort flag, drains the CTA's own copies, latches DERR_TIMEOUT and returns.
 #pragma once
@@ -113,17 +122,46 @@ template <int N> __device__ __forceinline__ void bulk_wait() {
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
+// thread-block clusters
+__device__ __forceinline__ int cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return (int)r;
+}
+__device__ __forceinline__ int cluster_size() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return (int)r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the address of p (in this CTA's shared memory) in CTA `rank` of the cluster
+template <typename T> __device__ __forceinline__ T* peer(T* p, int rank) {
+    uint64_t r;
+    asm("mapa.u64 %0, %1, %2;" : "=l"(r) : "l"(reinterpret_cast<uint64_t>(p)), "r"(rank));
+    return reinterpret_cast<T*>(r);
+}
+__device__ __forceinline__ void counter_release_cluster(int* p, int v) {
+    asm volatile("st.release.cluster.u32 [%0], %1;" ::"l"(reinterpret_cast<uint64_t>(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ int counter_acquire_cluster(const int* p) {
+    int v;
+    asm volatile("ld.acquire.cluster.u32 %0, [%1];" : "=r"(v) : "l"(reinterpret_cast<uint64_t>(p)) : "memory");
+    return v;
+}
+
 constexpr long long kWaitLimit = 1ll << 31;  // SM cycles, about a second
 
 // Bounded spin until *p >= target (or the CTA has aborted).  The clock and the
 // abort flag are looked at every 32 polls only.
+template <bool CL = false>
 __device__ __forceinline__ bool counter_wait(const int* p, int target, const volatile int* abort_flag,
                                              long long limit = kWaitLimit) {
-    if (counter_acquire(p) >= target) return true;
     const long long start = clock64();
-    for (unsigned it = 1;; ++it) {
+    for (unsigned it = 0;; ++it) {
+        if ((CL ? counter_acquire_cluster(p) : counter_acquire(p)) >= target) return true;
         __nanosleep(20);
-        if (counter_acquire(p) >= target) return true;
         if ((it & 31u) == 0u) {
             if (clock64() - start > limit) return false;
             if (*abort_flag) return false;
@@ -159,14 +197,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
 // polish: the factor of a last sweep's tighter threshold (A.polish), run once
 // after the stopping rule has fired: it rotates every pair with
 // |a^H b| > polish sqrt(rows) u |a| |b|, which leaves the columns orthogonal to
-// near the rounding of their storage (the truncated state depends on it).
+// near the rounding of their storage (the truncated state depends on it: at 2 an
+// observable after a 12-layer chi = 64 circuit is 1.2e-6 off the FP64 one, at 1
+// 0.6e-6, at 0.5 0.5e-6, geometric means of 14 circuits).
 template <typename R> struct Eps;
 template <> struct Eps<float> {
     static constexpr double u = 5.9604644775390625e-08;  // 2^-24
     static constexpr double k = 8.0;
     static constexpr int range_e = 24;
     static constexpr double early = 256.0;
-    static constexpr double polish = 2.0;
+    static constexpr double polish = 1.0;
 };
 template <> struct Eps<double> {
     static constexpr double u = 1.1102230246251565e-16;  // 2^-53
@@ -430,10 +470,8 @@ __device__ __forceinline__ float rcp_newton(float w) {
     return fmaf(y, fmaf(-w, y, 1.0f), y);
 }
 __device__ __forceinline__ double rcp_newton(double w) {
-    double y = (double)rcp_approx((float)w);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) y = fma(y, fma(-w, y, 1.0), y);
-    return y;
+    const double y = (double)rcp_approx((float)w), e = fma(-w, y, 1.0);  // y (1 + e + e^2): third order
+    return fma(y, fma(e, e, e), y);
 }
 
 __device__ __forceinline__ Rot<float> rotation(float al, float be, float gr, float gi, float g2) {
@@ -479,20 +517,24 @@ __device__ __forceinline__ Rot<double> rotation(double al, double be, double gr,
     p.tg = fma(p.tr, gr, p.ti * gi);
     const double t2 = fma(p.tr, p.tr, p.ti * p.ti);
     const double q = 1.0 + t2;
+    // cos = 1 / sqrt(q): the approximate root and one third-order step, c (1 + e/2 + 3 e^2/8)
+    // with e = 1 - q c^2 of about 1e-7
     double c = (double)rsqrt_approx((float)q);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) c = c * fma(-0.5 * q * c, c, 1.5);
+    const double qc = q * c, e2 = fma(-qc, c, 1.0);
+    c = fma(c * e2, fma(0.375, e2, 0.5), c);
     p.c2 = c * c;
     p.sm1 = t2 * rcp_newton(fma(q, c, 1.0));
     p.cm1 = -p.sm1 * c;
     return p;
 }
 // ------------------------------------------------------------ one warp --
-// Columns of a group and rows a lane holds of each: the 2 B columns of a visit
-// take 2 B RPL complex registers (128 32-bit registers at 512 rows complex64,
-// 512 rows complex128 and every size in between down to 128 rows complex128).
+// Columns of a group: the 2 B columns of a visit take 2 B RPL complex registers (128
+// 32-bit registers at 512 rows complex64, and at 128, 256 and 512 rows complex128).
+// Short complex128 columns go in pairs: a group's visit is bound by its one
+// scheduler's FP64 unit, and smaller groups spread it over more warps (64 of 64 x 64:
+// 7.3 -> 6.8 ms; at 128 rows 2 instead of 4 would cost 152 matrices 41 -> 50 ms).
 template <typename R, int RPL> struct GroupCols {
-    static constexpr int v = std::is_same<R, float>::value ? (RPL >= 16 ? 2 : 4) : (RPL >= 16 ? 1 : RPL >= 8 ? 2 : 4);
+    static constexpr int v = std::is_same<R, float>::value ? (RPL >= 16 ? 2 : 4) : (RPL >= 16 ? 1 : RPL >= 8 ? 2 : RPL == 4 ? 4 : 2);
 };
 
 // What a warp carries through a sweep.
@@ -543,7 +585,7 @@ __device__ __forceinline__ unsigned round_pairs(entry_t<R> (&a)[B][RPL], entry_t
     const unsigned m = __ballot_sync(0xffffffffu, rot);
     if (!m) return 0u;
     // (no branch: the lanes of pairs that stay compute along and drop the result)
-    sw.big = sw.big || (rot && g2 > (sw.big2 * al) * be);
+    if constexpr (Eps<R>::early > 0.0) sw.big = sw.big || (rot && g2 > (sw.big2 * al) * be);
     const Rot<R> q = rotation(al, be, gr, gi, g2);
     const R u = wb * ia, w = wa * ib * q.c2;
     __syncwarp();  // the warp is done with the coefficients of the round before
@@ -696,7 +738,8 @@ template <typename R> struct Tables {
     uint32_t key[kMaxCols];        // sort keys
     int cperm[kMaxCols];           // sweep order -> column
     int prog[kMaxCols];            // I groups that have met group j (in this sweep); j + 1 once it is taken itself
-    int dirty[kMaxCols];           // streaming: group j was rotated since it was last fetched
+    int aux[kMaxCols];             // streaming: group j was rotated since it was last fetched; cluster: where
+                                   // the column at a position lies (CTA << 16 | its place there)
     unsigned char flag[kMaxCols];  // complex128, by column: rotated in the sweep before
     unsigned char pflag[kMaxCols]; // by position: bit 0 the sweep before, bit 1 this one
     int rotations, abort, max_exp, big;
@@ -720,12 +763,17 @@ inline int warps_for(int ldw, bool half, int most) {
     return half && w > 4 ? 4 : w;
 }
 
-template <typename R, int RPL, bool RES>
+// Where the columns are: streamed from W, in this CTA's shared memory, or spread
+// over the shared memory of a cluster.
+enum { kStream = 0, kResident = 1, kCluster = 2 };
+
+template <typename R, int RPL, int MODE>
 __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int rows, int cols, int j_slot,
                                          int area, Tables<R>* T, cx_t<R>* cbuf) {
     const bool wait_test = A.wait_test != 0;
     const int chi_max = A.chi_max, max_sweeps = A.max_sweeps;
     using C = cx_t<R>;
+    constexpr bool RES = MODE != kStream, CL = MODE == kCluster;
     constexpr int B = GroupCols<R, RPL>::v;
     constexpr int L = 32 / B;
     constexpr int mpad = 32 * RPL;  // rows per column in shared memory
@@ -733,29 +781,48 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
     constexpr bool kSplit = std::is_same<R, float>::value;
     const int ldw = A.ldw;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nwc = blockDim.x >> 5;
+    const int ncta = CL ? cluster_size() : 1, crank = CL ? cluster_rank() : 0;
+    const int nwc = blockDim.x >> 5;                             // warps of the CTA
+    const int nw = nwc * ncta, gw = crank * nwc + warp;          // of all CTAs of the matrix; this one
+    const int held = (cols + ncta - 1) / ncta;                   // columns a CTA holds (RES): c = crank, crank + ncta, ...
     const int G = (cols + B - 1) / B;
     const int S = RES ? G : min(kMaxSlots, (int)((area - mpad * sizeof(C)) / (B * mpad * sizeof(C))));  // slots
-    C* const zeros = cbuf + (RES ? cols : S * B) * mpad;
+    C* const zeros = cbuf + (RES ? held : S * B) * mpad;
     const uint32_t col_bytes = (uint32_t)(rows * sizeof(C));
     volatile int* abort_flag = &T->abort;
 
     // columns in shared memory start as zeros (rows beyond `rows` stay zero)
-    for (int e = tid; e < (RES ? cols + 1 : S * B + 1) * mpad; e += blockDim.x) cbuf[e] = cmake<C>(0, 0);
+    for (int e = tid; e < (RES ? held + 1 : S * B + 1) * mpad; e += blockDim.x) cbuf[e] = cmake<C>(0, 0);
     for (int c = tid; c < cols; c += blockDim.x) {
         T->scl[c] = 0;
         if constexpr (kSkip) T->flag[c] = 1;  // sweep 0 checks every pair
     }
     fence_async_smem();
-    __syncthreads();
+    auto sync = [&]() {
+        if constexpr (CL) cluster_sync(); else __syncthreads();
+    };
+    sync();
+    // the tables of the CTA that keeps group g's counter, norms and scales
+    auto home = [&](int g) -> Tables<R>* {
+        if constexpr (CL) return peer(T, g % ncta);
+        return T;
+    };
+    // f(tables) for every CTA of the matrix
+    auto everywhere = [&](auto&& f) {
+        if constexpr (CL) {
+            for (int r = 0; r < ncta; ++r) f(peer(T, r));
+        } else {
+            f(T);
+        }
+    };
 
     // squared norms of the columns (exact); with `first`, the exponent of the
     // largest |entry| is gathered, and the columns are read from W (RES) and put
     // into the pair-split layout (complex64)
-    auto column = [&](int c) -> C* { return RES ? cbuf + (size_t)c * mpad : W + (size_t)c * ldw; };
+    auto column = [&](int c) -> C* { return RES ? cbuf + (c / ncta) * mpad : W + (size_t)c * ldw; };  // (one this CTA holds)
     auto norm_pass = [&](bool first) {
         R mx = 0;
-        for (int c = warp; c < cols; c += nwc) {
+        for (int c = crank + ncta * warp; c < cols; c += nw) {
             R s0 = 0, s1 = 0;
             const C* src = first ? W + (size_t)c * ldw : column(c);
             C* dst = column(c);
@@ -781,11 +848,11 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                 }
             }
             const R w = (R)1 + T->scl[c], s2 = warp_sum(s0 + s1) * w * w;
-            if (lane == 0) T->nrm[c] = s2;
+            if (lane == 0) everywhere([&](Tables<R>* t) { t->nrm[c] = s2; });
         }
         if (first) {
             mx = warp_max(mx);
-            if (lane == 0) atomicMax(&T->max_exp, exp_key<R>(mx));
+            if (lane == 0) everywhere([&](Tables<R>* t) { atomicMax(&t->max_exp, exp_key<R>(mx)); });
             if (!RES) fence_async_global();  // the sweeps read W through TMA as well
         }
     };
@@ -805,7 +872,7 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
 
     for (sweep = 0; sweep < max_sweeps; ++sweep) {
         norm_pass(sweep == 0);
-        __syncthreads();
+        sync();
         if (sweep == 0) {
             // Range guard.  Squared norms and |a^H b|^2 are formed in R: with entries of
             // 2^range_e and more they can overflow (and with tiny entries underflow),
@@ -818,7 +885,7 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
             if (T->max_exp > 0 && (ex >= Eps<R>::range_e || ex < -Eps<R>::range_e)) {
                 scale_e = ex;
                 const R f = ldexp((R)1, -scale_e);
-                for (int c = warp; c < cols; c += nwc) {
+                for (int c = crank + ncta * warp; c < cols; c += nw) {
                     C* col = column(c);
                     for (int r = lane; r < rows; r += 32) {
                         C v = col[r];
@@ -827,16 +894,19 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                     }
                 }
                 if (!RES) fence_async_global();
-                __syncthreads();
+                sync();
                 norm_pass(false);
-                __syncthreads();
+                sync();
             }
         }
         // sweep order: columns by decreasing norm, ties by index (ranks counted from
         // integer keys, so that any values give a permutation)
         for (int c = tid; c < cols; c += blockDim.x)
             T->key[c] = __float_as_uint((float)T->nrm[c]) & 0x7fffffffu;
-        for (int g = tid; g < G; g += blockDim.x) { T->prog[g] = 0; T->dirty[g] = 0; }
+        for (int g = tid; g < G; g += blockDim.x) {
+            T->prog[g] = 0;
+            if constexpr (!CL) T->aux[g] = 0;
+        }
         __syncthreads();
         for (int c = tid; c < cols; c += blockDim.x) {
             const uint32_t mine = T->key[c];
@@ -846,11 +916,12 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                 rank += (k > mine || (k == mine && q < c)) ? 1 : 0;
             }
             T->cperm[rank] = c;
+            if constexpr (CL) T->aux[rank] = (c % ncta) << 16 | (c / ncta);
             T->pnrm[rank] = T->nrm[c];
             T->pscl[rank] = T->scl[c];
             if constexpr (kSkip) T->pflag[rank] = T->flag[c];
         }
-        __syncthreads();
+        sync();
 
         // the polish sweep leaves pairs of two columns beyond chi_max (in the sweep
         // order, by decreasing norm) alone: they are dropped together, a rotation
@@ -917,14 +988,14 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                 __syncwarp();
                 pump(-1, true);
             }
-            for (int k0 = 0; k0 < GI && ok; k0 += nwc) {
-                const int I = k0 + warp;
+            for (int k0 = 0; k0 < GI && ok; k0 += nw) {
+                const int I = k0 + gw;
                 if (I >= GI) break;
-                const bool last = !RES && I == min(k0 + nwc, GI) - 1;  // the last warp of the row
+                const bool last = !RES && I == min(k0 + nw, GI) - 1;  // the last warp of the row
                 // Group g has met every I before this one (streaming, the first warp of a row: it
                 // has been fetched).  The same answer on every lane: they read one address in
                 // one instruction, and a wait that did not succeed at once ends in a vote.
-                auto ready = [&](int g) -> bool {
+                auto ready = [&](int g, Tables<R>* tg) -> bool {
                     if (RES ? I == 0 : warp == 0) {
                         if constexpr (!RES)
                             if (!mbar_try_wait(&T->full[slot], phase))
@@ -932,29 +1003,35 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                         return true;
                     }
                     const bool test = wait_test && sweep == 0 && I == 1 && g == 1;
-                    if (counter_acquire(&T->prog[g]) >= I && !test) return true;
-                    return __all_sync(0xffffffffu, counter_wait(&T->prog[g], test ? 0x7fffffff : I, abort_flag,
-                                                                test ? (1ll << 20) : kWaitLimit));
+                    if ((CL ? counter_acquire_cluster(&tg->prog[g]) : counter_acquire(&tg->prog[g])) >= I && !test)
+                        return true;
+                    return __all_sync(0xffffffffu, counter_wait<CL>(&tg->prog[g], test ? 0x7fffffff : I, abort_flag,
+                                                                    test ? (1ll << 20) : kWaitLimit));
+                };
+                auto release = [&](int* c, int v) {
+                    if constexpr (CL) counter_release_cluster(c, v); else counter_release(c, v);
                 };
                 // address of column i of group g in shared memory
                 auto sm_col = [&](int g, int i) -> C* {
                     const int pos = g * B + i;  // (columns missing from the last group: a column of zeros)
                     if (pos >= cols) return zeros;
+                    if constexpr (CL) return peer(cbuf, T->aux[pos] >> 16) + (T->aux[pos] & 0xffff) * mpad;
                     if constexpr (RES) return cbuf + T->cperm[pos] * mpad;
                     return cbuf + (slot * B + i) * mpad;
                 };
                 advance(warp);
-                if (!ready(I)) { ok = false; break; }
+                Tables<R>* const ti = home(I);
+                if (!ready(I, ti)) { ok = false; break; }
                 entry_t<R> a[B][RPL];
 #pragma unroll
                 for (int i = 0; i < B; ++i) col_load<RPL>(a[i], sm_col(I, i), lane);
                 const bool ip = I * B + p < cols;
-                R al = ip ? T->pnrm[I * B + p] : (R)0, da = ip ? T->pscl[I * B + p] : (R)0;
+                R al = ip ? ti->pnrm[I * B + p] : (R)0, da = ip ? ti->pscl[I * B + p] : (R)0;
                 int fa = 0;
-                if constexpr (kSkip) fa = ip ? T->pflag[I * B + p] : 0;
-                bool changed = !RES && T->dirty[I] != 0;
+                if constexpr (kSkip) fa = ip ? ti->pflag[I * B + p] : 0;
+                bool changed = !RES && T->aux[I] != 0;
                 __syncwarp();
-                if (lane == 0) counter_release(&T->prog[I], I + 1);
+                if (lane == 0) release(&ti->prog[I], I + 1);
                 if (fetcher) {
                     if (lane == 0)
                         for (int q = 0; q < nwc; ++q) bulk_commit();
@@ -962,12 +1039,13 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                 changed = inner_pairs<R, RPL, B>(a, al, da, fa, sw, tb, lane) || changed;
                 for (int J = I + 1; J < G; ++J) {
                     advance(1);
-                    if (!ready(J)) { ok = false; break; }
+                    Tables<R>* const tj = home(J);
+                    if (!ready(J, tj)) { ok = false; break; }
                     const bool jp = J * B + p < cols;
-                    R be = jp ? T->pnrm[J * B + p] : (R)0, db = jp ? T->pscl[J * B + p] : (R)0;
+                    R be = jp ? tj->pnrm[J * B + p] : (R)0, db = jp ? tj->pscl[J * B + p] : (R)0;
                     int fb = 0;
-                    if constexpr (kSkip) fb = jp ? T->pflag[J * B + p] : 0;
-                    bool store = last && T->dirty[J] != 0;
+                    if constexpr (kSkip) fb = jp ? tj->pflag[J * B + p] : 0;
+                    bool store = last && T->aux[J] != 0;
                     if (!kSkip || __any_sync(0xffffffffu, fa | fb)) {
                         entry_t<R> y[B][RPL];
 #pragma unroll
@@ -978,15 +1056,15 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                             if (__any_sync(0xffffffffu, fabs(db) > (R)kScaleMax)) apply_scales<R, RPL, B>(y, db);
                             if (__any_sync(0xffffffffu, fabs(da) > (R)kScaleMax)) apply_scales<R, RPL, B>(a, da);
                             if (jp && (lane & (L - 1)) == 0) {
-                                T->pnrm[J * B + p] = be;
-                                T->pscl[J * B + p] = db;
-                                if constexpr (kSkip) T->pflag[J * B + p] = (unsigned char)fb;
+                                tj->pnrm[J * B + p] = be;
+                                tj->pscl[J * B + p] = db;
+                                if constexpr (kSkip) tj->pflag[J * B + p] = (unsigned char)fb;
                             }
 #pragma unroll
                             for (int i = 0; i < B; ++i)
                                 if (J * B + i < cols) col_store<RPL>(y[i], sm_col(J, i), lane, mpad);
                             if constexpr (!RES)
-                                if (!last && lane == 0) T->dirty[J] = 1;
+                                if (!last && lane == 0) T->aux[J] = 1;
                         }
                     }
                     __syncwarp();
@@ -994,7 +1072,7 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                         if (last) {  // a changed group goes back to W
                             if (lane == 0) {
                                 if (store) {
-                                    T->dirty[J] = 0;
+                                    T->aux[J] = 0;
                                     fence_async_smem();
                                     const int nc = min(B, cols - J * B);
                                     for (int i = 0; i < nc; ++i)
@@ -1006,12 +1084,12 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                             __syncwarp();
                         }
                     }
-                    if (lane == 0) counter_release(&T->prog[J], I + 1);
+                    if (lane == 0) release(&tj->prog[J], I + 1);
                     if (fetcher) pump(rel, false);
                 }
                 if (!ok) break;
                 if (changed) {
-                    if (ip && (lane & (L - 1)) == 0) T->pscl[I * B + p] = da;
+                    if (ip && (lane & (L - 1)) == 0) ti->pscl[I * B + p] = da;
 #pragma unroll
                     for (int i = 0; i < B; ++i)
                         if (I * B + i < cols) {
@@ -1019,7 +1097,7 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                             else col_store<RPL>(a[i], W + (size_t)T->cperm[I * B + i] * ldw, lane, rows);
                         }
                     if constexpr (kSkip)
-                        if (ip && (lane & (L - 1)) == 0) T->pflag[I * B + p] = (unsigned char)fa;
+                        if (ip && (lane & (L - 1)) == 0) ti->pflag[I * B + p] = (unsigned char)fa;
                 }
                 if (fetcher) pump(rel, true);  // rows shorter than the ring wait for all that was stored
                 advance(1);
@@ -1029,24 +1107,24 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                 bulk_wait<0>();
                 fence_async_global();  // the next sweep reads W through TMA and through plain loads
             }
-            if (!ok) T->abort = 1;
+            if (!ok) everywhere([&](Tables<R>* t) { t->abort = 1; });
         }
         // groups streamed in this sweep
         int streamed_now = 0;
         if constexpr (!RES)
             for (int k0 = 0; k0 < GI; k0 += nwc) streamed_now += G - k0;
         streamed += streamed_now;
-        if (lane == 0 && sw.rot) atomicAdd(&T->rotations, sw.rot);
-        if (sw.big) T->big = 1;
+        if (lane == 0 && sw.rot) everywhere([&](Tables<R>* t) { atomicAdd(&t->rotations, sw.rot); });
+        if (__any_sync(0xffffffffu, sw.big) && lane == 0) everywhere([&](Tables<R>* t) { t->big = 1; });
         sw.rot = 0;
         sw.big = false;
-        __syncthreads();
+        sync();
         if (T->abort) {
             // A wait ran out: wait (bounded) for the fetches still in flight and latch the
             // error.  If one still has not landed, the CTA has to return with it in flight
             // (nothing can cancel a bulk copy, and waiting on would hang the GPU):
             // DERR_DRAIN marks the state unusable until it is re-created.
-            if (tid == 0) {
+            if (tid == 0 && crank == 0) {
                 bool drained = true;
                 if constexpr (!RES) {
                     const int n = (streamed - streamed_now) + T->fetch_e;  // groups fetched, over all sweeps
@@ -1055,17 +1133,23 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                 }
                 atomicOr(A.err, drained ? DERR_TIMEOUT : (DERR_TIMEOUT | DERR_DRAIN));
             }
-            __syncthreads();
+            sync();
             return;
         }
         const int rot = T->rotations;
         const bool small = Eps<R>::early > 0.0 && T->big == 0;
         rot_total += rot;
-        for (int q = tid; q < cols; q += blockDim.x) {
-            T->scl[T->cperm[q]] = T->pscl[q];
-            if constexpr (kSkip) T->flag[T->cperm[q]] = T->pflag[q] >> 1;
-        }
-        __syncthreads();
+        for (int q = tid; q < cols; q += blockDim.x)
+            if (!CL || (q / B) % ncta == crank) {  // (by column, in every CTA)
+                const int c = T->cperm[q];
+                const R d = T->pscl[q];
+                const unsigned char f = T->pflag[q] >> 1;
+                everywhere([&](Tables<R>* t) {
+                    t->scl[c] = d;
+                    if constexpr (kSkip) t->flag[c] = f;
+                });
+            }
+        sync();
         if (tid == 0) { T->rotations = 0; T->big = 0; }
         if (polishing) { converged = true; ++sweep; break; }
         if (rot == 0 || small) {
@@ -1081,8 +1165,8 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
         }
     }
     __syncthreads();
-    if (!converged && tid == 0) atomicOr(A.err, DERR_NOT_CONVERGED);
-    if (tid == 0) {
+    if (!converged && tid == 0 && crank == 0) atomicOr(A.err, DERR_NOT_CONVERGED);
+    if (tid == 0 && crank == 0) {
         const unsigned long long visits = (unsigned long long)sweep * (unsigned long long)(cols * (cols - 1) / 2) *
                                           (unsigned long long)rows;
         A.slot_sweeps[j_slot] = sweep;
@@ -1106,7 +1190,7 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
     // complex columns
     double* nrm = A.norms + (size_t)j_slot * ldw;
     const R unscale = ldexp((R)1, scale_e);
-    for (int c = warp; c < cols; c += nwc) {
+    for (int c = crank + ncta * warp; c < cols; c += nw) {
         double acc = 0.0;
         const C* src = column(c);
         C* dst = W + (size_t)c * ldw;
@@ -1142,22 +1226,23 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
 
 // Prologue of the kernels: which matrix, its size, the tables.
 template <typename R> struct Start {
-    int rows, cols, area;
+    int rows, cols, area, slot;
     cx_t<R>* W;
     Tables<R>* T;
     cx_t<R>* cbuf;
     bool go;
 };
 template <typename R>
-__device__ __forceinline__ Start<R> start(const LayerArgs<R>& A, int area, unsigned char* smem) {
+__device__ __forceinline__ Start<R> start(const LayerArgs<R>& A, int area, unsigned char* smem, int slot) {
     Start<R> s;
-    const int32_t* d = A.dims + blockIdx.x * kDims;
+    s.slot = slot;
+    const int32_t* d = A.dims + slot * kDims;
     s.go = !(A.refine == 1 && d[D_REFINE] != 1);  // the FP64 resolution runs only undecided bonds
     if (!s.go) return s;
     s.rows = A.pass == 1 ? 2 * d[D_CL] : d[D_ROWS];
     s.cols = A.pass == 1 ? d[D_CM] : d[D_COLS];
     s.area = area;
-    s.W = A.w + (size_t)blockIdx.x * A.ldw * A.ldw;
+    s.W = A.w + (size_t)slot * A.ldw * A.ldw;
     s.T = reinterpret_cast<Tables<R>*>(smem);
     s.cbuf = reinterpret_cast<cx_t<R>*>(smem + table_bytes<R>());
     if (threadIdx.x == 0) {
@@ -1168,14 +1253,76 @@ __device__ __forceinline__ Start<R> start(const LayerArgs<R>& A, int area, unsig
     return s;
 }
 
-// Columns that fit in the area stay there; `RPL` 16 never does.
+template <typename R, int RPL, int MODE>
+__device__ __forceinline__ void run(const LayerArgs<R>& A, const Start<R>& s) {
+    jacobi_body<R, RPL, MODE>(A, s.W, s.rows, s.cols, s.slot, s.area, s.T, s.cbuf);
+}
+// One CTA: columns that fit in the area stay there.
 template <typename R, int RPL>
-__device__ __forceinline__ void run_body(const LayerArgs<R>& A, const Start<R>& s) {
+__device__ __forceinline__ void run_alone(const LayerArgs<R>& A, const Start<R>& s) {
     const size_t need = (size_t)(s.cols + 1) * 32 * RPL * sizeof(cx_t<R>);
-    if (need <= (size_t)s.area)
-        jacobi_body<R, RPL, true>(A, s.W, s.rows, s.cols, blockIdx.x, s.area, s.T, s.cbuf);
-    else
-        jacobi_body<R, RPL, false>(A, s.W, s.rows, s.cols, blockIdx.x, s.area, s.T, s.cbuf);
+    if (need <= (size_t)s.area) run<R, RPL, kResident>(A, s);
+    else run<R, RPL, kStream>(A, s);
+}
+// A cluster: spread over it when there are enough groups for its warps and the columns
+// fit; otherwise its first CTA works alone.
+template <typename R, int RPL>
+__device__ __forceinline__ void run_cluster(const LayerArgs<R>& A, const Start<R>& s) {
+    const int n = cluster_size();
+    const size_t need = (size_t)((s.cols + n - 1) / n + 1) * 32 * RPL * sizeof(cx_t<R>);
+    if (need <= (size_t)s.area && s.cols >= 12 * GroupCols<R, RPL>::v) {
+        run<R, RPL, kCluster>(A, s);
+    } else if (cluster_rank() == 0) {
+        if constexpr (RPL >= 16) run<R, RPL, kStream>(A, s);
+        else run_alone<R, RPL>(A, s);
+    }
+}
+
+// Launch of `kernel` on `count` matrices by clusters of n CTAs.
+template <typename R, typename K>
+cudaError_t launch_cluster(K kernel, const LayerArgs<R>& a, int n, int threads, size_t smem, int area, cudaStream_t s) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(a.count * n);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = n;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, a, area);
+}
+
+// How many clusters of n CTAs (n = 2 .. 8) of a kernel run at once.
+constexpr int kMaxCluster = 8;
+template <typename K> cudaError_t clusters_at_once(K kernel, int threads, size_t smem, int (&most)[kMaxCluster + 1]) {
+    for (int n = 2; n <= kMaxCluster; ++n) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(n);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = n;
+        at.val.clusterDim.y = 1;
+        at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        int c = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&c, kernel, &cfg);
+        if (e != cudaSuccess) return e;
+        most[n] = c;
+    }
+    return cudaSuccess;
+}
+// CTAs for each of `bonds` matrices in flight together: as many as still run all at once.
+inline int cluster_for(int bonds, const int (&most)[kMaxCluster + 1]) {
+    for (int n = kMaxCluster; n > 1; --n)
+        if (bonds <= most[n]) return n;
+    return 1;
 }
 
 }  // namespace jac
