@@ -11,6 +11,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 #include <string>
 #include <type_traits>
@@ -51,6 +52,7 @@ struct ptebd_state {
     int ptsu_shortcut = 1;  // leave out the identity half-step after a layer on bonds 0, 2, 4, ... (see run_layer)
     int tensor_cores = 1;   // complex64 theta' on the tensor cores (ptebd_set_tensor_cores)
     int polish = 2;         // complex64 Jacobi polish sweep: 0 none, 1 gated SVDs, 2 gated and tSU, 3 tSU
+    char* host = nullptr;   // pinned, mapped: where small reads of the state land (owned)
     cudaStream_t body_stream = nullptr;  // captures the bodies of the FP64 pass's IF nodes (owned)
     // set once a device error says that a CTA returned with its own bulk copies still in
     // flight (DERR_DRAIN): the state and its workspace can no longer be trusted, and
@@ -62,6 +64,7 @@ struct ptebd_state {
         if (fork_ev) cudaEventDestroy(fork_ev);
         for (cudaStream_t x : aux) cudaStreamDestroy(x);
         if (body_stream) cudaStreamDestroy(body_stream);
+        if (host) cudaFreeHost(host);
     }
 };
 
@@ -659,13 +662,53 @@ int sync_and_check(ptebd_state* st) {
     return check_device_errors(st);
 }
 
-std::vector<int32_t> host_chi(ptebd_state* st, int* rc) {
+// Small reads of the state.  One kernel gathers the pieces and the error word into
+// pinned host memory and one synchronisation brings them, where a copy and a
+// synchronisation each took 39 us for the three of a Schmidt spectrum (reading
+// all of them took as long as the layers of a 128-site, chi = 64 step).
+struct Piece { const void* src; size_t bytes; };  // bytes a multiple of 4, src 4-byte aligned
+struct Pieces { const uint32_t* src[4]; uint32_t words[4]; };
+constexpr size_t kHostHead = 16;  // the error word, ahead of the pieces
+
+size_t host_bytes(const Layout& L) {  // the largest read: eps, nu and rank of every bond, or a Lambda and its length
+    const size_t n = (size_t)L.n_sites + 1;
+    return kHostHead + std::max(n * (2 * sizeof(double) + sizeof(int32_t)), (size_t)L.chip * sizeof(double) + 8) + 64;
+}
+
+__global__ void __launch_bounds__(256) k_read(Pieces p, const uint32_t* err, uint32_t* dst) {
+    if (threadIdx.x == 0) dst[0] = *err;
+    uint32_t* out = dst + kHostHead / 4;
+    for (int i = 0; i < 4; ++i) {
+        for (uint32_t w = threadIdx.x; w < p.words[i]; w += 256) out[w] = p.src[i][w];
+        out += p.words[i];
+    }
+}
+
+// The pieces, one behind the other, at *data (valid until the next read); `check`: a
+// latched device error is reported (and cleared) instead.
+int read_state(ptebd_state* st, std::initializer_list<Piece> pieces, const char** data, bool check = true) {
+    if (check && st->poisoned) return refuse_poisoned(st);
+    Pieces p{};
+    int n = 0;
+    for (const Piece& x : pieces) {
+        p.src[n] = static_cast<const uint32_t*>(x.src);
+        p.words[n++] = (uint32_t)(x.bytes / 4);
+    }
+    k_read<<<1, 256, 0, st->stream>>>(p, at<uint32_t>(st->mem, st->L.off_err), reinterpret_cast<uint32_t*>(st->host));
+    CUDA_TRY(st, cudaGetLastError());
+    CUDA_TRY(st, cudaStreamSynchronize(st->stream));
+    uint32_t err;
+    std::memcpy(&err, st->host, sizeof err);
+    *data = st->host + kHostHead;
+    return check && err ? check_device_errors(st) : PTEBD_OK;
+}
+
+// Every bond dimension (n_sites + 1 of them), after the errors of the work before.
+std::vector<int32_t> host_chi(ptebd_state* st, int* rc, bool check = true) {
     std::vector<int32_t> chi((size_t)st->L.n_sites + 1);
-    *rc = PTEBD_OK;
-    cudaError_t e = cudaMemcpyAsync(chi.data(), at<int32_t>(st->mem, st->L.off_chi), chi.size() * sizeof(int32_t),
-                                    cudaMemcpyDeviceToHost, st->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st->stream);
-    if (e != cudaSuccess) *rc = set_err(st, PTEBD_ERR_CUDA, "reading bond dimensions failed: %s", cudaGetErrorString(e));
+    const char* d;
+    *rc = read_state(st, {{at<int32_t>(st->mem, st->L.off_chi), chi.size() * sizeof(int32_t)}}, &d, check);
+    if (!*rc) std::memcpy(chi.data(), d, chi.size() * sizeof(int32_t));
     return chi;
 }
 
@@ -975,6 +1018,12 @@ int ptebd_create(const ptebd_config* cfg, void* state_mem, size_t state_bytes, v
     st->slots = slots;
     st->stream = static_cast<cudaStream_t>(stream);
     cudaGetDevice(&st->device);
+    if (cudaHostAlloc(reinterpret_cast<void**>(&st->host), host_bytes(L), cudaHostAllocMapped) != cudaSuccess) {
+        cudaGetLastError();
+        st->host = nullptr;
+        delete st;
+        return PTEBD_ERR_MEMORY;
+    }
     cudaError_t e = cfg->precision == PTEBD_FP64 ? jacobi_prepare<double>() : jacobi_prepare<float>();
     if (e == cudaSuccess) e = cfg->precision == PTEBD_FP64 ? orth_prepare<double>() : orth_prepare<float>();
     if (e == cudaSuccess && cfg->precision == PTEBD_MIXED) e = theta_tc_prepare();
@@ -1241,10 +1290,8 @@ int ptebd_sync(ptebd_state* st) {
 
 int ptebd_norm(ptebd_state* st, double* out) {
     if (!st || !out) return set_err(st, PTEBD_ERR_INVALID, "null argument");
-    int rc = sync_and_check(st);
-    if (rc) return rc;
     double v[2];
-    rc = contract(st, st, v);
+    const int rc = contract(st, st, v);
     if (rc) return rc;
     *out = std::sqrt(std::max(v[0], 0.0));
     return PTEBD_OK;
@@ -1254,32 +1301,24 @@ int ptebd_overlap(ptebd_state* a, ptebd_state* b, double out[2]) {
     if (!a || !b || !out) return set_err(a, PTEBD_ERR_INVALID, "null argument");
     if (a->L.n_sites != b->L.n_sites) return set_err(a, PTEBD_ERR_INVALID, "different n_sites");
     if (a->L.chip != b->L.chip) return set_err(a, PTEBD_ERR_INVALID, "overlap needs equal chi_max padding");
-    int rc = sync_and_check(a);
-    if (rc) return rc;
-    if ((rc = sync_and_check(b))) return rc;
     return contract(a, b, out);
 }
 
 int ptebd_expect(ptebd_state* st, int32_t site, const double* op, double out[2]) {
     if (!st || !op || !out) return set_err(st, PTEBD_ERR_INVALID, "null argument");
     if (site < 0 || site >= st->L.n_sites) return set_err(st, PTEBD_ERR_INVALID, "site out of range");
-    int rc = sync_and_check(st);
-    if (rc) return rc;
     return expectation(st, site, 1, op, out);
 }
 
 int ptebd_expect2(ptebd_state* st, int32_t site, const double* op, double out[2]) {
     if (!st || !op || !out) return set_err(st, PTEBD_ERR_INVALID, "null argument");
     if (site < 0 || site >= st->L.n_sites - 1) return set_err(st, PTEBD_ERR_INVALID, "site out of range");
-    int rc = sync_and_check(st);
-    if (rc) return rc;
     return expectation(st, site, 2, op, out);
 }
 
 int ptebd_get_chi(ptebd_state* st, int32_t* chi_out) {
     if (!st || !chi_out) return set_err(st, PTEBD_ERR_INVALID, "null argument");
-    int rc = sync_and_check(st);
-    if (rc) return rc;
+    int rc;
     std::vector<int32_t> chi = host_chi(st, &rc);
     if (rc) return rc;
     for (int b = 0; b < st->L.n_sites - 1; ++b) chi_out[b] = chi[b + 1];
@@ -1289,14 +1328,13 @@ int ptebd_get_chi(ptebd_state* st, int32_t* chi_out) {
 int ptebd_get_lambda(ptebd_state* st, int32_t bond, double* out, int32_t* k) {
     if (!st || !out) return set_err(st, PTEBD_ERR_INVALID, "null argument");
     if (bond < 0 || bond > st->L.n_sites - 2) return set_err(st, PTEBD_ERR_INVALID, "bond out of range");
-    int rc = sync_and_check(st);
+    const char* d;
+    const size_t row = (size_t)st->L.chip * sizeof(double);
+    const int rc = read_state(st, {{lam_ptr(st, bond), row}, {at<int32_t>(st->mem, st->L.off_chi) + bond + 1, 4}}, &d);
     if (rc) return rc;
     int32_t kk;
-    CUDA_TRY(st, cudaMemcpyAsync(&kk, at<int32_t>(st->mem, st->L.off_chi) + bond + 1, sizeof kk, cudaMemcpyDeviceToHost,
-                                 st->stream));
-    CUDA_TRY(st, cudaStreamSynchronize(st->stream));
-    CUDA_TRY(st, cudaMemcpyAsync(out, lam_ptr(st, bond), (size_t)kk * sizeof(double), cudaMemcpyDeviceToHost, st->stream));
-    CUDA_TRY(st, cudaStreamSynchronize(st->stream));
+    std::memcpy(&kk, d + row, sizeof kk);
+    std::memcpy(out, d, (size_t)kk * sizeof(double));
     if (k) *k = kk;
     return PTEBD_OK;
 }
@@ -1304,8 +1342,7 @@ int ptebd_get_lambda(ptebd_state* st, int32_t bond, double* out, int32_t* k) {
 int ptebd_get_site(ptebd_state* st, int32_t site, int32_t* chi_l, int32_t* chi_r, double* gamma_out) {
     if (!st) return PTEBD_ERR_INVALID;
     if (site < 0 || site >= st->L.n_sites) return set_err(st, PTEBD_ERR_INVALID, "site out of range");
-    int rc = sync_and_check(st);
-    if (rc) return rc;
+    int rc;
     std::vector<int32_t> chi = host_chi(st, &rc);
     if (rc) return rc;
     const int cl = chi[site], cr = chi[site + 1];
@@ -1352,7 +1389,7 @@ int ptebd_set_site(ptebd_state* st, int32_t site, int32_t chi_l, int32_t chi_r, 
     if (!st || !gamma) return set_err(st, PTEBD_ERR_INVALID, "null argument");
     if (site < 0 || site >= st->L.n_sites) return set_err(st, PTEBD_ERR_INVALID, "site out of range");
     int rc;
-    std::vector<int32_t> chi = host_chi(st, &rc);
+    std::vector<int32_t> chi = host_chi(st, &rc, false);
     if (rc) return rc;
     if (chi[site] != chi_l || chi[site + 1] != chi_r)
         return set_err(st, PTEBD_ERR_SHAPE, "site %d: got %dx%d, bonds say %dx%d", site, chi_l, chi_r, chi[site],
@@ -1378,11 +1415,11 @@ int ptebd_set_site(ptebd_state* st, int32_t site, int32_t chi_l, int32_t chi_r, 
 
 int ptebd_trunc_error(ptebd_state* st, double* eps_total, double* log_nu_total) {
     if (!st) return PTEBD_ERR_INVALID;
-    int rc = sync_and_check(st);
+    const char* d;
+    const int rc = read_state(st, {{at<double>(st->mem, st->L.off_totals), 2 * sizeof(double)}}, &d);
     if (rc) return rc;
-    double t[8];
-    CUDA_TRY(st, cudaMemcpyAsync(t, at<double>(st->mem, st->L.off_totals), sizeof t, cudaMemcpyDeviceToHost, st->stream));
-    CUDA_TRY(st, cudaStreamSynchronize(st->stream));
+    double t[2];
+    std::memcpy(t, d, sizeof t);
     if (eps_total) *eps_total = t[0];
     if (log_nu_total) *log_nu_total = t[1];
     return PTEBD_OK;
@@ -1390,13 +1427,15 @@ int ptebd_trunc_error(ptebd_state* st, double* eps_total, double* log_nu_total) 
 
 int ptebd_bond_stats(ptebd_state* st, double* eps, double* nu, int32_t* rank_in) {
     if (!st) return PTEBD_ERR_INVALID;
-    int rc = sync_and_check(st);
-    if (rc) return rc;
     const size_t nb = (size_t)st->L.n_sites - 1;
-    if (eps) CUDA_TRY(st, cudaMemcpyAsync(eps, at<double>(st->mem, st->L.off_bond_eps), nb * sizeof(double), cudaMemcpyDeviceToHost, st->stream));
-    if (nu) CUDA_TRY(st, cudaMemcpyAsync(nu, at<double>(st->mem, st->L.off_bond_nu), nb * sizeof(double), cudaMemcpyDeviceToHost, st->stream));
-    if (rank_in) CUDA_TRY(st, cudaMemcpyAsync(rank_in, at<int32_t>(st->mem, st->L.off_bond_rank), nb * sizeof(int32_t), cudaMemcpyDeviceToHost, st->stream));
-    CUDA_TRY(st, cudaStreamSynchronize(st->stream));
+    const char* d;
+    const int rc = read_state(st, {{at<double>(st->mem, st->L.off_bond_eps), nb * sizeof(double)},
+                                   {at<double>(st->mem, st->L.off_bond_nu), nb * sizeof(double)},
+                                   {at<int32_t>(st->mem, st->L.off_bond_rank), nb * sizeof(int32_t)}}, &d);
+    if (rc) return rc;
+    if (eps) std::memcpy(eps, d, nb * sizeof(double));
+    if (nu) std::memcpy(nu, d + nb * sizeof(double), nb * sizeof(double));
+    if (rank_in) std::memcpy(rank_in, d + 2 * nb * sizeof(double), nb * sizeof(int32_t));
     return PTEBD_OK;
 }
 
@@ -1615,8 +1654,7 @@ int ptebd_sample(ptebd_state* st, int32_t n_samples, const double* uniforms, int
     if (n_samples == 0) return PTEBD_OK;
     if (workspace && ((uintptr_t)workspace & 255))
         return set_err(st, PTEBD_ERR_INVALID, "the sampling workspace must be 256-byte aligned");
-    int rc = sync_and_check(st);
-    if (rc) return rc;
+    int rc;
     std::vector<int32_t> chi = host_chi(st, &rc);
     if (rc) return rc;
     const int N = st->L.n_sites, chip = st->L.chip;
@@ -1666,13 +1704,11 @@ int ptebd_sample(ptebd_state* st, int32_t n_samples, const double* uniforms, int
 
 int ptebd_svd_sweeps(ptebd_state* st, int32_t* sweeps, int32_t* layers) {
     if (!st) return PTEBD_ERR_INVALID;
-    int rc = sync_and_check(st);
+    const size_t nb = (size_t)st->L.n_sites - 1;
+    const char* d;
+    const int rc = read_state(st, {{at<int32_t>(st->mem, st->L.off_bond_sweeps), nb * sizeof(int32_t)}}, &d);
     if (rc) return rc;
-    if (sweeps) {
-        CUDA_TRY(st, cudaMemcpyAsync(sweeps, at<int32_t>(st->mem, st->L.off_bond_sweeps),
-                                     (size_t)(st->L.n_sites - 1) * sizeof(int32_t), cudaMemcpyDeviceToHost, st->stream));
-        CUDA_TRY(st, cudaStreamSynchronize(st->stream));
-    }
+    if (sweeps) std::memcpy(sweeps, d, nb * sizeof(int32_t));
     if (layers) *layers = st->layers;
     return PTEBD_OK;
 }
