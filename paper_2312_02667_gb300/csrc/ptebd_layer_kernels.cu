@@ -276,7 +276,7 @@ __device__ int op_schmidt_rank(const double* g) {
     return rank;
 }
 
-// grid (count), 512 threads.  norms[] holds the FP64 column norms of the
+// grid (count), ldw threads (64 at least).  norms[] holds the FP64 column norms of the
 // rotated matrix (= the singular values, unsorted).
 // With a.resolve > a.thr_rel (the complex64 pass of a state with FP64
 // resolution), singular values <= resolve * sigma_1 are not trusted: the kept
@@ -287,34 +287,61 @@ __device__ int op_schmidt_rank(const double* g) {
 // marked (dims D_REFINE = 1) and left alone: the FP64 pass recomputes it.
 template <typename R>
 __global__ void __launch_bounds__(512) k_truncate(LayerArgs<R> a) {
-    constexpr int NS = 512;
-    __shared__ double key[NS];
-    __shared__ int idx[NS];
-    __shared__ double red[NS];
+    constexpr int kMax = 512;
+    __shared__ double key[kMax];
+    __shared__ int idx[kMax];
+    __shared__ double red[2][kMax / 32];
     __shared__ int kept_sh, kept_hi_sh, rmax_sh;
+    __shared__ double scale_sh, eps_sh, nu_sh;
     const int j = blockIdx.x, t = threadIdx.x;
     int32_t* d = a.dims + j * kDims;
     if (a.refine == 1 && d[D_REFINE] != 1) return;
     const int ncols = d[D_COLS];
     const int b = d[D_BOND];
     const double* nrm = a.norms + (size_t)j * a.ldw;
-    key[t] = (t < ncols) ? nrm[t] : -1.0;
-    idx[t] = t;
-    __syncthreads();
-    // bitonic sort, descending by value, ascending index on ties
-    for (int size = 2; size <= NS; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            const int p = t ^ stride;
-            if (p > t) {
-                const bool desc = (t & size) == 0;
-                const double kt = key[t], kp = key[p];
-                const int it = idx[t], ip = idx[p];
-                const bool t_first = (kt > kp) || (kt == kp && it < ip);
-                if (desc ? !t_first : t_first) {
-                    key[t] = kp; key[p] = kt; idx[t] = ip; idx[p] = it;
+    // descending by value, ascending index on ties (norms compared as integers, so that any
+    // values, a NaN too, give a permutation)
+    auto before = [](double x, int i, double y, int q) {
+        const long long u = __double_as_longlong(x) & 0x7fffffffffffffffll,
+                        v = __double_as_longlong(y) & 0x7fffffffffffffffll;
+        return u > v || (u == v && i < q);
+    };
+    if (ncols <= 128) {
+        // few columns: every thread counts its rank (a bitonic sort's steps cost a barrier each:
+        // 33 us for the 512-wide one this was at every size, 6 us now at 32 columns)
+        const double mine = t < ncols ? nrm[t] : 0.0;
+        key[t] = mine;
+        __syncthreads();
+        int rank = 0;
+        if (t < ncols)
+            for (int q = 0; q < ncols; ++q) rank += before(key[q], q, mine, t) ? 1 : 0;
+        __syncthreads();
+        if (t < ncols) {
+            key[rank] = mine;
+            idx[rank] = t;
+        }
+        __syncthreads();
+    } else {
+        int ns = 256;
+        while (ns < ncols) ns <<= 1;
+        if (t < ns) {
+            key[t] = t < ncols ? nrm[t] : 0.0;
+            idx[t] = t < ncols ? t : kMax + t;  // (padding: zeros behind every column)
+        }
+        __syncthreads();
+        for (int size = 2; size <= ns; size <<= 1) {
+            for (int stride = size >> 1; stride > 0; stride >>= 1) {
+                const int p = t ^ stride;
+                if (t < ns && p > t) {
+                    const bool desc = (t & size) == 0;
+                    const double kt = key[t], kp = key[p];
+                    const int it = idx[t], ip = idx[p];
+                    if (desc != before(kt, it, kp, ip)) {
+                        key[t] = kp; key[p] = kt; idx[t] = ip; idx[p] = it;
+                    }
                 }
+                __syncthreads();
             }
-            __syncthreads();
         }
     }
     const double smax = key[0];
@@ -362,36 +389,48 @@ __global__ void __launch_bounds__(512) k_truncate(LayerArgs<R> a) {
         }
         k = max(1, k_hi);
     }
-    // FP64 weights: total and dropped, fixed-order tree sums
+    // FP64 weights: total and dropped, fixed-order sums
     const double w = (t < ncols) ? key[t] * key[t] : 0.0;
-    red[t] = w;
-    __syncthreads();
-    for (int s = NS / 2; s > 0; s >>= 1) {
-        if (t < s) red[t] += red[t + s];
-        __syncthreads();
+    double wt = w, wd = t >= k ? w : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        wt += __shfl_xor_sync(0xffffffffu, wt, o);
+        wd += __shfl_xor_sync(0xffffffffu, wd, o);
     }
-    const double total = red[0];
-    __syncthreads();
-    red[t] = (t >= k) ? w : 0.0;
-    __syncthreads();
-    for (int s = NS / 2; s > 0; s >>= 1) {
-        if (t < s) red[t] += red[t + s];
-        __syncthreads();
+    if ((t & 31) == 0) {
+        red[0][t >> 5] = wt;
+        red[1][t >> 5] = wd;
     }
-    const double dropped = red[0];
-    double eps = (a.eps_mode == PTEBD_EPS_ABSOLUTE) ? dropped : dropped / total;
-    double nu = 1.0;
-    if (a.stabilise) {
-        if (eps < 1.0) {
-            nu = 1.0 / sqrt(1.0 - eps);
-        } else if (t == 0) {
-            atomicOr(a.err, DERR_EPS);
+    __syncthreads();
+    // one warp for the rest: a square root or a quotient costs the FP64 pipe as much in
+    // every warp that takes it
+    if (t < 32) {
+        double total = t < (int)(blockDim.x >> 5) ? red[0][t] : 0.0, dropped = t < (int)(blockDim.x >> 5) ? red[1][t] : 0.0;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            total += __shfl_xor_sync(0xffffffffu, total, o);
+            dropped += __shfl_xor_sync(0xffffffffu, dropped, o);
+        }
+        const double eps = (a.eps_mode == PTEBD_EPS_ABSOLUTE) ? dropped : dropped / total;
+        double nu = 1.0;
+        if (a.stabilise) {
+            if (eps < 1.0) {
+                nu = 1.0 / sqrt(1.0 - eps);
+            } else if (t == 0) {
+                atomicOr(a.err, DERR_EPS);
+            }
+        }
+        if (t == 0) {
+            // Lambda_b <- nu S_kept, or nu S_kept / |S| (the Schmidt reading; tSU keeps S)
+            scale_sh = (a.stabilise && a.eps_mode == PTEBD_EPS_SCHMIDT) ? nu / sqrt(total) : nu;
+            eps_sh = eps;
+            nu_sh = nu;
         }
     }
-    // Lambda_b <- nu S_kept, or nu S_kept / |S| (the Schmidt reading; tSU keeps S)
-    const double lam_scale = (a.stabilise && a.eps_mode == PTEBD_EPS_SCHMIDT) ? nu / sqrt(total) : nu;
+    __syncthreads();
+    const double lam_scale = scale_sh, eps = eps_sh, nu = nu_sh;
     double* lam_b = a.lam + (size_t)(b + 1) * a.chip;
-    for (int q = t; q < a.chip; q += NS) lam_b[q] = (q < k) ? lam_scale * key[q] : 0.0;
+    for (int q = t; q < a.chip; q += blockDim.x) lam_b[q] = (q < k) ? lam_scale * key[q] : 0.0;
     if (t < k) {
         a.sig[(size_t)j * a.ldw + t] = key[t];
         a.perm[(size_t)j * a.ldw + t] = idx[t];
@@ -753,13 +792,20 @@ __global__ void k_add_partials(const double* partials, int k, double* totals) {
 }
 
 // -------------------------------------------------------------- launchers --
+// The complex64 products go to the tensor cores from this padded bond dimension on.
+// At 64 both ways take the same time (theta' and Gamma of a 128-site step 0.35 and
+// 0.34 ms), at 128 the tensor cores save 0.4 of a 200-site step's 30 ms, and their
+// truncating accumulation is the larger error (the discarded weights of a 12-layer
+// chi = 64 circuit 4.5e-6 off FP64 against 1.5e-6).  At 256 they take 3.7 ms a gated
+// theta' of 511 bonds, the CUDA cores 9.9.
+constexpr int kTensorCoreChi = 256;
 template <typename R, typename G> cudaError_t launch_theta(const LayerArgs<R>& a, cudaStream_t s) {
     // tensor_cores 1: gated stages; 2: the tSU steps as well.  On a tSU step the
     // accumulation's residual shrinkage (about 2e-7 per product) is not
     // renormalised away, and over the bonds of a PtSU step it moves the norm of
     // the state: 5.4e-4 at N = 1024, chi = 256.
     if constexpr (std::is_same<R, float>::value)
-        if (a.tensor_cores && (a.mode == 0 || a.tensor_cores == 2) && a.chip >= 64 && a.refine == 0)
+        if (a.tensor_cores && (a.mode == 0 || a.tensor_cores == 2) && a.chip >= kTensorCoreChi && a.refine == 0)
             return launch_theta_tc(a, s);
     const int tiles = (a.chip + 31) / 32;
     dim3 grid(tiles, tiles, a.count);
@@ -767,7 +813,7 @@ template <typename R, typename G> cudaError_t launch_theta(const LayerArgs<R>& a
     return cudaGetLastError();
 }
 template <typename R> cudaError_t launch_truncate(const LayerArgs<R>& a, cudaStream_t s) {
-    k_truncate<R><<<a.count, 512, 0, s>>>(a);
+    k_truncate<R><<<a.count, a.ldw < 64 ? 64 : a.ldw, 0, s>>>(a);
     return cudaGetLastError();
 }
 template <typename R, typename G> cudaError_t launch_gamma(const LayerArgs<R>& a, cudaStream_t s) {
@@ -777,7 +823,7 @@ template <typename R, typename G> cudaError_t launch_gamma(const LayerArgs<R>& a
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if constexpr (std::is_same<R, float>::value)
-        if (a.tensor_cores && (a.mode == 0 || a.tensor_cores == 2) && a.chip >= 64 && a.refine == 0)
+        if (a.tensor_cores && (a.mode == 0 || a.tensor_cores == 2) && a.chip >= kTensorCoreChi && a.refine == 0)
             return launch_gamma_gemm_tc(a, s);
     const int tiles = (a.chip + 31) / 32;
     dim3 g2(tiles, tiles, 2 * a.count);
@@ -792,7 +838,7 @@ template <typename R, typename G> cudaError_t launch_xform(const LayerArgs<R>& a
 }
 template <typename R> cudaError_t launch_proj(const LayerArgs<R>& a, cudaStream_t s) {
     if constexpr (std::is_same<R, float>::value)
-        if (a.tensor_cores == 2 && a.chip >= 64 && a.refine == 0) return launch_proj_tc(a, s);
+        if (a.tensor_cores == 2 && a.chip >= kTensorCoreChi && a.refine == 0) return launch_proj_tc(a, s);
     dim3 grid((2 * a.chip + 31) / 32, (a.chip + 31) / 32, a.count);
     k_proj<R><<<grid, 256, 0, s>>>(a);
     return cudaGetLastError();
