@@ -20,9 +20,10 @@
 //
 // What bounds it: the FP64 pipe (2 fused multiply-adds per SM and cycle: a 64 x 64 x
 // 64 complex product is 3.5 us of the whole chip) and, at small bond dimensions, the
-// latency of a launch.  Hence 8 x 8 output tiles of 64 threads: chi = 64 gives 128
+// latency of a launch.  Hence 8 x 8 output tiles of 128 threads: chi = 64 gives 128
 // tiles a side (32 x 32 tiles of 256 threads kept 4 of 152 SMs busy at 65 us a
-// product), and two launches a step for both sides instead of five for one.
+// product; 64 threads leave two of an SM's four FP64 units idle), and two launches
+// a step for both sides instead of five for one.
 #include <cmath>
 
 #include "ptebd_internal.h"
@@ -48,16 +49,18 @@ __device__ __forceinline__ double unit_scale(const unsigned long long* bits) {
     return __longlong_as_double((long long)(2046 - e) << 52);
 }
 
-constexpr int kTile = 8, kChunk = 32, kThreads = 64;
+constexpr int kTile = 8, kChunk = 64, kThreads = 128;
 
-// grid (ceil(max m / 8), ceil(max n / 8), problems), 64 threads, one output each.
-// The chunk of k after the one being multiplied is already on its way from memory.
+// grid (ceil(max m / 8), ceil(max n / 8), problems), 128 threads: each half of them takes
+// one half of every chunk of k for the tile's 64 outputs, so that all four schedulers'
+// FP64 units work.  The chunk after the one being multiplied is already on its way
+// from memory.
 __global__ void __launch_bounds__(kThreads) k_zmm(ZmmBatch batch) {
     const Zmm& q = batch.p[blockIdx.z];
     const int i0 = blockIdx.x * kTile, j0 = blockIdx.y * kTile;
     if (i0 >= q.m || j0 >= q.n) return;
     __shared__ double2 as[kChunk][kTile + 1], bs[kChunk][kTile + 1];
-    const int t = threadIdx.x, ti = t & 7, tj = t >> 3;
+    const int t = threadIdx.x, half = t >> 6, ti = t & 7, tj = (t >> 3) & 7;
     const int per = (q.k + kChunk - 1) / kChunk, chunks = per * q.segments;
     double2 ra[4], rb[4];
     // element e of a chunk: the index that is contiguous in memory runs fastest
@@ -67,7 +70,7 @@ __global__ void __launch_bounds__(kThreads) k_zmm(ZmmBatch batch) {
         for (int u = 0; u < 4; ++u) {
             const int e = t + u * kThreads;
             int kk, ii;
-            if (q.op_a == ZMM_C) { kk = e & 31; ii = e >> 5; } else { ii = e & 7; kk = e >> 3; }
+            if (q.op_a == ZMM_C) { kk = e & 63; ii = e >> 6; } else { ii = e & 7; kk = e >> 3; }
             const int k = k0 + kk, i = i0 + ii;
             double2 v = make_double2(0.0, 0.0);
             if (k < q.k && i < q.m) {
@@ -78,7 +81,7 @@ __global__ void __launch_bounds__(kThreads) k_zmm(ZmmBatch batch) {
             }
             ra[u] = v;
             int kb, jj;
-            if (q.op_b == ZMM_T) { jj = e & 7; kb = e >> 3; } else { kb = e & 31; jj = e >> 5; }
+            if (q.op_b == ZMM_T) { jj = e & 7; kb = e >> 3; } else { kb = e & 63; jj = e >> 6; }
             const int k2 = k0 + kb, j = j0 + jj;
             double2 w = make_double2(0.0, 0.0);
             if (k2 < q.k && j < q.n) {
@@ -92,8 +95,8 @@ __global__ void __launch_bounds__(kThreads) k_zmm(ZmmBatch batch) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int e = t + u * kThreads;
-            if (q.op_a == ZMM_C) as[e & 31][e >> 5] = ra[u]; else as[e >> 3][e & 7] = ra[u];
-            if (q.op_b == ZMM_T) bs[e >> 3][e & 7] = rb[u]; else bs[e & 31][e >> 5] = rb[u];
+            if (q.op_a == ZMM_C) as[e & 63][e >> 6] = ra[u]; else as[e >> 3][e & 7] = ra[u];
+            if (q.op_b == ZMM_T) bs[e >> 3][e & 7] = rb[u]; else bs[e & 63][e >> 6] = rb[u];
         }
     };
     double2 acc = make_double2(0.0, 0.0);
@@ -102,26 +105,27 @@ __global__ void __launch_bounds__(kThreads) k_zmm(ZmmBatch batch) {
         put();
         __syncthreads();
         if (c + 1 < chunks) fetch(c + 1);
-        const int seg = c >= per ? 1 : 0, depth = min(kChunk, q.k - (c - seg * per) * kChunk);
-        if (depth == kChunk) {
+        // (a chunk is zero beyond the end of k; a short one is halved evenly)
+        const int seg = c >= per ? 1 : 0, depth = (min(kChunk, q.k - (c - seg * per) * kChunk) + 1) / 2;
+        const double2 (*pa)[kTile + 1] = as + half * depth, (*pb)[kTile + 1] = bs + half * depth;
 #pragma unroll 8
-            for (int kk = 0; kk < kChunk; ++kk) {
-                const double2 x = as[kk][ti], y = bs[kk][tj];
-                acc.x = fma(x.x, y.x, acc.x); acc.y = fma(x.x, y.y, acc.y);
-                acc.x = fma(-x.y, y.y, acc.x); acc.y = fma(x.y, y.x, acc.y);
-            }
-        } else {
-            for (int kk = 0; kk < depth; ++kk) {
-                const double2 x = as[kk][ti], y = bs[kk][tj];
-                acc.x = fma(x.x, y.x, acc.x); acc.y = fma(x.x, y.y, acc.y);
-                acc.x = fma(-x.y, y.y, acc.x); acc.y = fma(x.y, y.x, acc.y);
-            }
+        for (int kk = 0; kk < depth; ++kk) {
+            const double2 x = pa[kk][ti], y = pb[kk][tj];
+            acc.x = fma(x.x, y.x, acc.x); acc.y = fma(x.x, y.y, acc.y);
+            acc.x = fma(-x.y, y.y, acc.x); acc.y = fma(x.y, y.x, acc.y);
         }
         __syncthreads();
     }
+    double2* other = &as[0][0];
+    if (half) other[t & 63] = acc;
+    __syncthreads();
+    if (!half) {
+        acc.x += other[t].x;
+        acc.y += other[t].y;
+    }
     const int i = i0 + ti, j = j0 + tj;
     double big = 0.0;
-    if (i < q.m && j < q.n) {
+    if (!half && i < q.m && j < q.n) {
         double f = unit_scale(q.scale_a) * unit_scale(q.scale_b);
         if (q.rowscale) f *= q.rowscale[i];
         if (q.colscale) f *= q.colscale[j];
@@ -130,7 +134,7 @@ __global__ void __launch_bounds__(kThreads) k_zmm(ZmmBatch batch) {
         static_cast<double2*>(q.c)[(size_t)j * q.ldc + i] = acc;
         big = fmax(fabs(acc.x), fabs(acc.y));
     }
-    if (q.largest) {
+    if (q.largest && !half) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
         if ((t & 31) == 0) atomicMax(q.largest, (unsigned long long)__double_as_longlong(big));
