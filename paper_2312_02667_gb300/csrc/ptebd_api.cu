@@ -769,6 +769,7 @@ void left_step(ptebd_state* a, ptebd_state* b, const std::vector<int32_t>& ca, c
     q.a[1] = gptr(a, s, 1);
     q.b[1] = t1;
     q.segments = 2;
+    q.hermitian = a == b;
     q.rowscale = lam_ptr(a, s);
     q.colscale = lam_ptr(b, s);
     q.largest = next;
@@ -788,6 +789,7 @@ void right_step(ptebd_state* a, ptebd_state* b, const std::vector<int32_t>& ca, 
     q.a[1] = t1;
     q.b[1] = gptr(b, s, 1);
     q.segments = 2;
+    q.hermitian = a == b;
     q.rowscale = lam_ptr(a, s - 1);
     q.colscale = lam_ptr(b, s - 1);
     q.largest = next;

@@ -20,7 +20,7 @@
 //
 // What bounds it: the FP64 pipe (2 fused multiply-adds per SM and cycle: a 64 x 64 x
 // 64 complex product is 3.5 us of the whole chip) and, at small bond dimensions, the
-// latency of a launch.  Hence 8 x 8 output tiles of 128 threads: chi = 64 gives 128
+// latency of a launch.  Hence 4 x 8 output tiles of 128 threads: chi = 64 gives 256
 // tiles a side (32 x 32 tiles of 256 threads kept 4 of 152 SMs busy at 65 us a
 // product; 64 threads leave two of an SM's four FP64 units idle), and two launches
 // a step for both sides instead of five for one.
@@ -49,28 +49,32 @@ __device__ __forceinline__ double unit_scale(const unsigned long long* bits) {
     return __longlong_as_double((long long)(2046 - e) << 52);
 }
 
-constexpr int kTile = 8, kChunk = 64, kThreads = 128;
+constexpr int kTileM = 4, kTileN = 8, kChunk = 64, kThreads = 128;
 
-// grid (ceil(max m / 8), ceil(max n / 8), problems), 128 threads: each half of them takes
-// one half of every chunk of k for the tile's 64 outputs, so that all four schedulers'
+// grid (ceil(max m / 4), ceil(max n / 8), problems), 128 threads: each warp takes a
+// quarter of every chunk of k for the tile's 32 outputs, so that all four schedulers'
 // FP64 units work.  The chunk after the one being multiplied is already on its way
-// from memory.
+// from memory.  A Hermitian result is worked out on and above its diagonal.  The
+// launches of a chain are programmatic ones, without an explicit trigger: the next
+// one is set up as this one ends (8.1 -> 6.9 ms of measurements at N = 128, chi = 64);
+// triggered early, waiting blocks of the launches to come fill some of the SMs and
+// the next one's work piles up on the others (13.8 ms).
 __global__ void __launch_bounds__(kThreads) k_zmm(ZmmBatch batch) {
     const Zmm& q = batch.p[blockIdx.z];
-    const int i0 = blockIdx.x * kTile, j0 = blockIdx.y * kTile;
-    if (i0 >= q.m || j0 >= q.n) return;
-    __shared__ double2 as[kChunk][kTile + 1], bs[kChunk][kTile + 1];
-    const int t = threadIdx.x, half = t >> 6, ti = t & 7, tj = (t >> 3) & 7;
+    const int i0 = blockIdx.x * kTileM, j0 = blockIdx.y * kTileN;
+    if (i0 >= q.m || j0 >= q.n || (q.hermitian && i0 >= j0 + kTileN)) return;
+    __shared__ double2 as[kChunk][kTileM + 1], bs[kChunk][kTileN + 1];
+    const int t = threadIdx.x, quarter = t >> 5, ti = t & 3, tj = (t >> 2) & 7;
     const int per = (q.k + kChunk - 1) / kChunk, chunks = per * q.segments;
-    double2 ra[4], rb[4];
+    double2 ra[2], rb[4];
     // element e of a chunk: the index that is contiguous in memory runs fastest
     auto fetch = [&](int c) {
         const int seg = c >= per ? 1 : 0, k0 = (c - seg * per) * kChunk;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 2; ++u) {
             const int e = t + u * kThreads;
             int kk, ii;
-            if (q.op_a == ZMM_C) { kk = e & 63; ii = e >> 6; } else { ii = e & 7; kk = e >> 3; }
+            if (q.op_a == ZMM_C) { kk = e & 63; ii = e >> 6; } else { ii = e & 3; kk = e >> 2; }
             const int k = k0 + kk, i = i0 + ii;
             double2 v = make_double2(0.0, 0.0);
             if (k < q.k && i < q.m) {
@@ -80,12 +84,16 @@ __global__ void __launch_bounds__(kThreads) k_zmm(ZmmBatch batch) {
                 if (q.kscale) { v.x *= q.kscale[k]; v.y *= q.kscale[k]; }
             }
             ra[u] = v;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int e = t + u * kThreads;
             int kb, jj;
             if (q.op_b == ZMM_T) { jj = e & 7; kb = e >> 3; } else { kb = e & 63; jj = e >> 6; }
-            const int k2 = k0 + kb, j = j0 + jj;
+            const int k = k0 + kb, j = j0 + jj;
             double2 w = make_double2(0.0, 0.0);
-            if (k2 < q.k && j < q.n) {
-                const size_t at = q.op_b == ZMM_T ? (size_t)k2 * q.ldb + j : (size_t)j * q.ldb + k2;
+            if (k < q.k && j < q.n) {
+                const size_t at = q.op_b == ZMM_T ? (size_t)k * q.ldb + j : (size_t)j * q.ldb + k;
                 w = entry(q.b[seg], at, q.b32);
             }
             rb[u] = w;
@@ -93,21 +101,26 @@ __global__ void __launch_bounds__(kThreads) k_zmm(ZmmBatch batch) {
     };
     auto put = [&]() {
 #pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int e = t + u * kThreads;
+            if (q.op_a == ZMM_C) as[e & 63][e >> 6] = ra[u]; else as[e >> 2][e & 3] = ra[u];
+        }
+#pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int e = t + u * kThreads;
-            if (q.op_a == ZMM_C) as[e & 63][e >> 6] = ra[u]; else as[e >> 3][e & 7] = ra[u];
             if (q.op_b == ZMM_T) bs[e >> 3][e & 7] = rb[u]; else bs[e & 63][e >> 6] = rb[u];
         }
     };
     double2 acc = make_double2(0.0, 0.0);
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // everything before this launch is complete and visible
     fetch(0);
     for (int c = 0; c < chunks; ++c) {
         put();
         __syncthreads();
         if (c + 1 < chunks) fetch(c + 1);
-        // (a chunk is zero beyond the end of k; a short one is halved evenly)
-        const int seg = c >= per ? 1 : 0, depth = (min(kChunk, q.k - (c - seg * per) * kChunk) + 1) / 2;
-        const double2 (*pa)[kTile + 1] = as + half * depth, (*pb)[kTile + 1] = bs + half * depth;
+        // (a chunk is zero beyond the end of k; a short one is quartered evenly)
+        const int seg = c >= per ? 1 : 0, depth = (min(kChunk, q.k - (c - seg * per) * kChunk) + 3) / 4;
+        const double2 (*pa)[kTileM + 1] = as + quarter * depth, (*pb)[kTileN + 1] = bs + quarter * depth;
 #pragma unroll 8
         for (int kk = 0; kk < depth; ++kk) {
             const double2 x = pa[kk][ti], y = pb[kk][tj];
@@ -116,28 +129,34 @@ __global__ void __launch_bounds__(kThreads) k_zmm(ZmmBatch batch) {
         }
         __syncthreads();
     }
-    double2* other = &as[0][0];
-    if (half) other[t & 63] = acc;
+    double2* other = &as[0][0];  // (3 x 32 of its 320 entries)
+    if (quarter) other[t - 32] = acc;
     __syncthreads();
-    if (!half) {
-        acc.x += other[t].x;
-        acc.y += other[t].y;
+    if (quarter) return;
+#pragma unroll
+    for (int h = 0; h < 3; ++h) {
+        acc.x += other[32 * h + t].x;
+        acc.y += other[32 * h + t].y;
     }
     const int i = i0 + ti, j = j0 + tj;
     double big = 0.0;
-    if (!half && i < q.m && j < q.n) {
+    if (i < q.m && j < q.n) {
         double f = unit_scale(q.scale_a) * unit_scale(q.scale_b);
         if (q.rowscale) f *= q.rowscale[i];
         if (q.colscale) f *= q.colscale[j];
         acc.x *= f;
         acc.y *= f;
-        static_cast<double2*>(q.c)[(size_t)j * q.ldc + i] = acc;
+        if (!q.hermitian || i <= j) {
+            if (q.hermitian && i == j) acc.y = 0.0;
+            q.c[(size_t)j * q.ldc + i] = acc;
+            if (q.hermitian && i < j) q.c[(size_t)i * q.ldc + j] = make_double2(acc.x, -acc.y);
+        }
         big = fmax(fabs(acc.x), fabs(acc.y));
     }
-    if (q.largest && !half) {
+    if (q.largest) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
-        if ((t & 31) == 0) atomicMax(q.largest, (unsigned long long)__double_as_longlong(big));
+        if (t == 0) atomicMax(q.largest, (unsigned long long)__double_as_longlong(big));
     }
 }
 
@@ -243,9 +262,16 @@ cudaError_t launch_zmm(const ZmmBatch& b, int n, cudaStream_t s) {
         c = b.p[i].n > c ? b.p[i].n : c;
     }
     if (m <= 0 || c <= 0) return cudaSuccess;
-    dim3 grid((m + kTile - 1) / kTile, (c + kTile - 1) / kTile, n);
-    k_zmm<<<grid, kThreads, 0, s>>>(b);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((m + kTileM - 1) / kTileM, (c + kTileN - 1) / kTileN, n);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_zmm, b);
 }
 
 cudaError_t launch_chain_start(double2* e, double2* f, unsigned long long* largest, int n, cudaStream_t s) {

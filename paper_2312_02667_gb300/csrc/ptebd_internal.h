@@ -167,6 +167,7 @@ struct Zmm {
     unsigned long long* largest;  // gathers the bits of the largest modulus of C (or null)
     int m, n, k, segments, lda, ldb, ldc, op_a, op_b;  // op_a: N, C, J; op_b: N, T
     bool a32, b32;
+    bool hermitian;  // C is Hermitian (m = n): its entries below the diagonal are taken from those above
 };
 struct ZmmBatch { Zmm p[8]; };
 cudaError_t launch_zmm(const ZmmBatch& b, int n, cudaStream_t s);
