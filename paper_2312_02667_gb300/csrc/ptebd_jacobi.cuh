@@ -62,6 +62,8 @@
 // abort flag, drains the CTA's own copies, latches DERR_TIMEOUT and returns.
 #pragma once
 #include <cmath>
+#include <map>
+#include <mutex>
 #include <type_traits>
 
 #include "ptebd_internal.h"
@@ -534,7 +536,7 @@ __device__ __forceinline__ Rot<double> rotation(double al, double be, double gr,
 // scheduler's FP64 unit, and smaller groups spread it over more warps (64 of 64 x 64:
 // 7.3 -> 6.8 ms; at 128 rows 2 instead of 4 would cost 152 matrices 41 -> 50 ms).
 template <typename R, int RPL> struct GroupCols {
-    static constexpr int v = std::is_same<R, float>::value ? (RPL >= 16 ? 2 : 4) : (RPL >= 16 ? 1 : RPL >= 8 ? 2 : RPL == 4 ? 4 : 2);
+    static constexpr int v = std::is_same<R, float>::value ? (RPL >= 12 ? 2 : 4) : (RPL >= 12 ? 1 : RPL >= 6 ? 2 : RPL == 4 ? 4 : 2);
 };
 
 // What a warp carries through a sweep.
@@ -1273,7 +1275,7 @@ __device__ __forceinline__ void run_cluster(const LayerArgs<R>& A, const Start<R
     if (need <= (size_t)s.area && s.cols >= 12 * GroupCols<R, RPL>::v) {
         run<R, RPL, kCluster>(A, s);
     } else if (cluster_rank() == 0) {
-        if constexpr (RPL >= 16) run<R, RPL, kStream>(A, s);
+        if constexpr (RPL >= 12) run<R, RPL, kStream>(A, s);
         else run_alone<R, RPL>(A, s);
     }
 }
@@ -1317,6 +1319,25 @@ template <typename K> cudaError_t clusters_at_once(K kernel, int threads, size_t
         most[n] = c;
     }
     return cudaSuccess;
+}
+struct MostClusters { int n[kMaxCluster + 1]; };
+// The same, found on first use (zeros where the kernel cannot be launched so).
+template <typename R>
+const MostClusters& most_clusters(void (*kernel)(LayerArgs<R>, int)) {
+    static std::mutex mu;
+    static std::map<const void*, MostClusters> found;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = found.find(reinterpret_cast<const void*>(kernel));
+    if (it == found.end()) {
+        MostClusters m{};
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
+            clusters_at_once(kernel, 256, kSmemMax, m.n) != cudaSuccess) {
+            cudaGetLastError();
+            m = MostClusters{};
+        }
+        it = found.emplace(reinterpret_cast<const void*>(kernel), m).first;
+    }
+    return it->second;
 }
 // CTAs for each of `bonds` matrices in flight together: as many as still run all at once.
 inline int cluster_for(int bonds, const int (&most)[kMaxCluster + 1]) {

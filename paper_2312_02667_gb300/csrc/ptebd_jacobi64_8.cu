@@ -1,0 +1,8 @@
+#include "ptebd_jacobi64.cuh"
+
+namespace ptebd {
+namespace jac {
+template cudaError_t prepare64<8>();
+template cudaError_t launch64<8>(const LayerArgs<double>&, cudaStream_t);
+}  // namespace jac
+}  // namespace ptebd

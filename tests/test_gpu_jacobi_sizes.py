@@ -1,5 +1,5 @@
 """The Jacobi SVD kernel at the sizes where its choices change: rows per lane
-(32, 64, 128, 256, 512 rows), matrices that stay in shared memory and matrices
+(32, 64, 96, 128, 192, 256, 384, 512 rows), matrices that stay in shared memory and matrices
 streamed through it, column counts that leave a partial last group, fewer
 groups than warps, and rank-deficient and graded columns, through svd_batched
 against LAPACK in complex128."""
@@ -9,8 +9,8 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 # (rows, cols): the edges of each row class, one past them, and thin matrices of each
-SIZES = [(2, 1), (6, 5), (32, 32), (34, 33), (64, 64), (64, 3), (66, 65), (98, 98), (102, 102), (128, 128), (128, 9),
-         (130, 127), (200, 130), (256, 103), (256, 105), (256, 256), (258, 50), (258, 255), (300, 111), (512, 17),
+SIZES = [(2, 1), (6, 5), (32, 32), (34, 33), (64, 64), (64, 3), (66, 65), (96, 95), (98, 98), (102, 102), (128, 128), (128, 9),
+         (130, 127), (192, 190), (194, 60), (200, 130), (256, 103), (256, 105), (256, 256), (258, 50), (258, 255), (300, 111), (384, 100), (386, 90), (512, 17),
          (512, 210)]
 U = {"mixed": 2.0 ** -24, "fp64": 2.0 ** -53}
 K = {"mixed": 8.0, "fp64": 4.0}  # the rotation threshold: |a^H b| <= K sqrt(rows) u |a| |b|
