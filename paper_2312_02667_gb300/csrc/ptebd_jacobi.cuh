@@ -471,8 +471,10 @@ __device__ __forceinline__ float rcp_newton(float w) {
     const float y = rcp_approx(w);
     return fmaf(y, fmaf(-w, y, 1.0f), y);
 }
+__device__ __forceinline__ float cut(double x, int k);
+__device__ __forceinline__ double widen(float x, int k);
 __device__ __forceinline__ double rcp_newton(double w) {
-    const double y = (double)rcp_approx((float)w), e = fma(-w, y, 1.0);  // y (1 + e + e^2): third order
+    const double y = widen(rcp_approx(cut(w, 0)), 0), e = fma(-w, y, 1.0);  // y (1 + e + e^2): third order
     return fma(y, fma(e, e, e), y);
 }
 
@@ -495,38 +497,73 @@ __device__ __forceinline__ Rot<float> rotation(float al, float be, float gr, flo
     p.cm1 = -p.sm1 * c;
     return p;
 }
-// complex128: tan(angle) e^{i arg g} is worked out in FP32 from values scaled by
-// a power of two (a tangent that is 1e-7 off leaves the pair orthogonal to
-// 1e-7 of its cos, which the next sweep's quadratic convergence does not notice),
-// since the FP64 square root and division cost more than the pair's dot product
-// there; cos is then taken from that same tangent in FP64, so that the rotation
-// is unitary to FP64 rounding.
-__device__ __forceinline__ Rot<double> rotation(double al, double be, double gr, double gi, double) {
-    const double big = fmax(al, be);
-    const int e = (__double2hiint(big) >> 20) & 0x7ff;
-    const int ie = 2046 - e;  // exponent field of 2^(1023 - e)
-    const double s = __hiloint2double((ie < 1 ? 1 : ie) << 20, 0);
+// complex128.  The FP64 unit takes 64 cycles for one instruction of a warp, and the
+// parameters of a round are worked out by every lane, so what need not be FP64 is
+// done with integers and in FP32:
+//   - the threshold test and tan(angle) e^{i arg g}: from FP32 values made by scaling
+//     with powers of two (a tangent that is 1e-7 off leaves the pair orthogonal to
+//     1e-7 of its cos, which the next sweep's quadratic convergence does not notice);
+//   - tan |g|, which updates the tracked norms: 1e-7 of it matters only in early sweeps;
+//   - conversions, scaling and comparisons of magnitudes: on the bits.
+// cos is taken from the rounded tangent in FP64, so that the rotation is unitary to
+// FP64 rounding.  50 FP64 instructions a round instead of 77.
+__device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }  // biased
+// x 2^k as FP32, truncated (0 below the normal range; NaN for an infinity or NaN)
+__device__ __forceinline__ float cut(double x, int k) {
+    const int hi = __double2hiint(x), e = ((hi >> 20) & 0x7ff) - 896 + k;
+    const uint32_t bits = ((uint32_t)hi & 0x80000000u) | ((uint32_t)e << 23) | (((uint32_t)hi & 0xfffffu) << 3) |
+                          ((uint32_t)__double2loint(x) >> 29);
+    if ((hi & 0x7ff00000) == 0x7ff00000) return __int_as_float(0x7fffffff);
+    return e < 1 || exponent(x) == 0 ? 0.0f : e > 254 ? __int_as_float(0x7f7fffff) : __uint_as_float(bits);
+}
+// x 2^k (x normal or 0)
+__device__ __forceinline__ double widen(float x, int k) {
+    const uint32_t b = __float_as_uint(x);
+    const int e = (int)((b >> 23) & 255u);
+    if (e == 0 || e + 896 + k < 1) return 0.0;
+    return __hiloint2double((int)((b & 0x80000000u) | ((uint32_t)(e + 896 + k) << 20) | ((b & 0x7fffffu) >> 3)),
+                            (int)(b << 29));
+}
+// |g|^2 > tol2 al be
+__device__ __forceinline__ bool over_threshold(double al, double be, double gr, double gi, float tol2) {
+    const int ea = exponent(al), eb = exponent(be);
+    const int sum = ea + eb - 2046, h = sum >> 1;  // g is scaled by about 1 / sqrt(al be)
+    const float x = cut(gr, -h), y = cut(gi, -h);
+    const float a = cut(al, 1023 - ea), b = cut(be, 1023 - eb);  // in [1, 2)
+    return ea > 0 && eb > 0 && fmaf(x, x, y * y) > tol2 * a * ((sum & 1) ? b + b : b);
+}
+struct Rot64 { double tr, ti, tg, c, c2, sq, cm1, sm1; };  // sq = 1/cos
+__device__ __forceinline__ Rot64 rotation64(double al, double be, double gr, double gi) {
+    const int ea = exponent(al), eb = exponent(be), e = (ea > eb ? ea : eb) - 1023;
     const double d = be - al;
-    const float df = (float)(d * s), grf = (float)(gr * s), gif = (float)(gi * s);
+    const float df = cut(d, -e), grf = cut(gr, -e), gif = cut(gi, -e);
     const float g2 = fmaf(grf, grf, gif * gif);
     const float h = fmaf(df, df, 4.0f * g2);
     const float root = h > 0.0f ? h * rsqrtf(h) : 0.0f;
     float f = __fdividef(2.0f, fabsf(df) + root);
-    if (d < 0.0) f = -f;
-    Rot<double> p;
-    p.tr = (double)(f * grf);
-    p.ti = (double)(f * gif);
-    p.tg = fma(p.tr, gr, p.ti * gi);
-    const double t2 = fma(p.tr, p.tr, p.ti * p.ti);
-    const double q = 1.0 + t2;
+    if (__double2hiint(d) < 0) f = -f;
+    Rot64 p;
+    p.tr = widen(f * grf, 0);
+    p.ti = widen(f * gif, 0);
+    p.tg = widen(f * g2, e);
+    if (__any_sync(0xffffffffu, ea > eb + 100 || eb > ea + 100)) {
+        // (lengths 1e15 apart and more: g may leave the FP32 range; the tangent is g / d)
+        if (ea > eb + 100 || eb > ea + 100) {
+            p.tr = gr / d;
+            p.ti = gi / d;
+            p.tg = fma(p.tr, gr, p.ti * gi);
+        }
+    }
+    const double t2 = fma(p.tr, p.tr, p.ti * p.ti), q = 1.0 + t2;
     // cos = 1 / sqrt(q): the approximate root and one third-order step, c (1 + e/2 + 3 e^2/8)
     // with e = 1 - q c^2 of about 1e-7
-    double c = (double)rsqrt_approx((float)q);
-    const double qc = q * c, e2 = fma(-qc, c, 1.0);
-    c = fma(c * e2, fma(0.375, e2, 0.5), c);
-    p.c2 = c * c;
-    p.sm1 = t2 * rcp_newton(fma(q, c, 1.0));
-    p.cm1 = -p.sm1 * c;
+    const double c0 = widen(rsqrt_approx(cut(q, 0)), 0);
+    const double qc = q * c0, e2 = fma(-qc, c0, 1.0);
+    p.c = fma(c0 * e2, fma(0.375, e2, 0.5), c0);
+    p.c2 = p.c * p.c;
+    p.sq = q * p.c;
+    p.sm1 = t2 * rcp_newton(1.0 + p.sq);
+    p.cm1 = -p.sm1 * p.c;
     return p;
 }
 // ------------------------------------------------------------ one warp --
@@ -542,73 +579,118 @@ template <typename R, int RPL> struct GroupCols {
 // What a warp carries through a sweep.
 template <typename R> struct Sweep {
     R tol2, big2;
+    float tol2f;
     bool big = false;  // this lane's pair was rotated with cos^2 >= big2
     int rot = 0;       // rotations of this warp
 };
 
+// A column as the lanes of its lane group hold it: true squared norm, scale minus 1,
+// the scale's reciprocal, and (complex128) whether it was rotated, bit 0 in the sweep
+// before and bit 1 in this one.
+template <typename R> struct Lane {
+    R n, d, i;
+    int f;
+    __device__ __forceinline__ R w() const { return (R)1 + d; }
+    __device__ __forceinline__ bool far() const {  // the scale has moved by 2^-6
+        if constexpr (std::is_same<R, float>::value) return fabs(d) > (R)(1.0 / 64);
+        return (__double2hiint(d) & 0x7fffffff) >= 0x3f900000;
+    }
+    __device__ __forceinline__ void move(int src) {  // to the column of lane src
+        n = __shfl_sync(0xffffffffu, n, src);
+        d = __shfl_sync(0xffffffffu, d, src);
+        if constexpr (!std::is_same<R, float>::value) {
+            i = __shfl_sync(0xffffffffu, i, src);
+            f = __shfl_sync(0xffffffffu, f, src);
+        }
+    }
+};
+
 // One round of B disjoint pairs (a[i], y[(i + r) mod B]).  Lane group p holds
-// al, da, fa of column p of a and be, db, fb of column (p + r) mod B of y: true
-// squared norm, scale minus 1, and (complex128) whether the column was rotated
-// in this sweep or the one before.  Pairs of two columns with neither flag set
-// met in the sweep before as the same two vectors and were orthogonal: their
-// dot product is left out (on the FP64 pipe it costs a third of a rotation, and
-// late sweeps are mostly such checks).  Returns the mask of lanes whose pair
-// rotated.
+// column p of a as ca and column (p + r) mod B of y as cy.  complex128: pairs of two
+// columns with no flag set met in the sweep before as the same two vectors and
+// were orthogonal: their dot product is left out (late sweeps are mostly such
+// checks).  Returns the mask of lanes whose pair rotated.
 template <typename R, int RPL, int B, int r>
-__device__ __forceinline__ unsigned round_pairs(entry_t<R> (&a)[B][RPL], entry_t<R> (&y)[B][RPL], R& al, R& da, int& fa,
-                                                R& be, R& db, int& fb, bool pair_ok, Sweep<R>& sw, Coef<R>* tb, int lane) {
-    constexpr bool kSkip = std::is_same<R, double>::value;
+__device__ __forceinline__ unsigned round_pairs(entry_t<R> (&a)[B][RPL], entry_t<R> (&y)[B][RPL], Lane<R>& ca,
+                                                Lane<R>& cy, Sweep<R>& sw, Coef<R>* tb, int lane) {
+    constexpr bool k64 = std::is_same<R, double>::value;
     constexpr int L = 32 / B;
     const int p = lane / L;
     R vr[B], vi[B];
     unsigned need = 0xffffffffu;
-    if constexpr (kSkip) {
-        need = __ballot_sync(0xffffffffu, pair_ok && (fa | fb));
+    if constexpr (k64) {
+        need = __ballot_sync(0xffffffffu, ca.f | cy.f);
         if (!need) return 0u;
     }
 #pragma unroll
     for (int i = 0; i < B; ++i) {
         vr[i] = 0;
         vi[i] = 0;
-        if (!kSkip || ((need >> (i * L)) & 1u)) col_dot<RPL>(a[i], y[(i + r) % B], vr[i], vi[i]);
+        if (!k64 || ((need >> (i * L)) & 1u)) col_dot<RPL>(a[i], y[(i + r) % B], vr[i], vi[i]);
     }
-    const R wa = (R)1 + da, wb = (R)1 + db;
-    const R ia = rcp_newton(wa), ib = rcp_newton(wb);
+    const R wa = ca.w(), wb = cy.w();
+    if constexpr (!k64) {
+        ca.i = rcp_newton(wa);
+        cy.i = rcp_newton(wb);
+    }
     R gr, gi;
     reduce_pairs<R, B>(vr, vi, lane, gr, gi);
     const R sc = wa * wb;
     gr *= sc;
     gi *= sc;
-    const R g2 = gr * gr + gi * gi;
-    // al, be >= 0 (a tracked norm that shrinks a lot is recomputed from its
+    // a.n, b.n >= 0 (a tracked norm that shrinks a lot is recomputed from its
     // column), so a zero column (g = 0) or a non-finite value fails this test and
     // is left alone
-    const bool rot = pair_ok && g2 > (sw.tol2 * al) * be;
+    const R al = ca.n, be = cy.n;
+    R g2 = 0;
+    bool rot;
+    if constexpr (k64) {
+        rot = over_threshold(al, be, gr, gi, sw.tol2f);
+    } else {
+        g2 = gr * gr + gi * gi;
+        rot = g2 > (sw.tol2 * al) * be;
+    }
     const unsigned m = __ballot_sync(0xffffffffu, rot);
     if (!m) return 0u;
     // (no branch: the lanes of pairs that stay compute along and drop the result)
-    if constexpr (Eps<R>::early > 0.0) sw.big = sw.big || (rot && g2 > (sw.big2 * al) * be);
-    const Rot<R> q = rotation(al, be, gr, gi, g2);
-    const R u = wb * ia, w = wa * ib * q.c2;
+    R tr, ti, kr, ki, al2, be2;
+    if constexpr (k64) {
+        const Rot64 q = rotation64(al, be, gr, gi);
+        const double u = wb * ca.i, w = (wa * cy.i) * q.c2;
+        tr = q.tr * u; ti = q.ti * u; kr = q.tr * w; ki = q.ti * w;
+        al2 = al - q.tg;
+        be2 = be + q.tg;
+        const double da = ca.d + fma(ca.d, q.cm1, q.cm1), db = cy.d + fma(cy.d, q.sm1, q.sm1);
+        const double ia = ca.i * q.sq, ib = cy.i * q.c;
+        if (rot) { ca.d = da; ca.i = ia; cy.d = db; cy.i = ib; ca.f |= 2; cy.f |= 2; }
+    } else {
+        if constexpr (Eps<R>::early > 0.0) sw.big = sw.big || (rot && g2 > (sw.big2 * al) * be);
+        const Rot<R> q = rotation(al, be, gr, gi, g2);
+        const R u = wb * ca.i, w = wa * cy.i * q.c2;
+        tr = q.tr * u; ti = q.ti * u; kr = q.tr * w; ki = q.ti * w;
+        al2 = al - q.tg;
+        be2 = be + q.tg;
+        const R cm1 = rot ? q.cm1 : (R)0, sm1 = rot ? q.sm1 : (R)0;
+        ca.d = ca.d + fma(ca.d, cm1, cm1);
+        cy.d = cy.d + fma(cy.d, sm1, sm1);
+    }
     __syncwarp();  // the warp is done with the coefficients of the round before
     // short columns: every pair of the round is sheared, a pair that stays by zero
     // (cheaper than a branch per pair); long ones: only the pairs that rotate
-    constexpr bool kAll = RPL <= 4 && !kSkip;
+    constexpr bool kAll = RPL <= 4 && !k64;
     if ((kAll || rot) && (lane & (L - 1)) == 0)
-        tb[p].set(rot ? q.tr * u : (R)0, rot ? q.ti * u : (R)0, rot ? q.tr * w : (R)0, rot ? q.ti * w : (R)0);
-    const R al2 = rot ? al - q.tg : al, be2 = rot ? be + q.tg : be;
-    const R cm1 = rot ? q.cm1 : (R)0, sm1 = rot ? q.sm1 : (R)0;
+        tb[p].set(rot ? tr : (R)0, rot ? ti : (R)0, rot ? kr : (R)0, rot ? ki : (R)0);
     // a norm that lost most of its size (cancellation in the update) is taken from its column
-    const bool shrunk = rot && !(al2 > (R)0.125 * al && be2 > (R)0.125 * be);
-    const bool sa = !(al2 > (R)0.125 * al), sb = !(be2 > (R)0.125 * be);
-    al = al2;
-    be = be2;
-    da = da + fma(da, cm1, cm1);
-    db = db + fma(db, sm1, sm1);
-    if constexpr (kSkip) {
-        fa |= rot ? 2 : 0;
-        fb |= rot ? 2 : 0;
+    bool sa, sb;
+    if constexpr (k64) {  // by exponents: less than an eighth, or negative
+        sa = __double2hiint(al2) < __double2hiint(al) - (3 << 20);
+        sb = __double2hiint(be2) < __double2hiint(be) - (3 << 20);
+    } else {
+        sa = !(al2 > (R)0.125 * al);
+        sb = !(be2 > (R)0.125 * be);
     }
+    const bool shrunk = rot && (sa || sb);
+    if (rot) { ca.n = al2; cy.n = be2; }
     __syncwarp();
     sw.rot += __popc(m) / L;
 #pragma unroll
@@ -620,11 +702,11 @@ __device__ __forceinline__ unsigned round_pairs(entry_t<R> (&a)[B][RPL], entry_t
         for (int i = 0; i < B; ++i) {
             if ((ma >> (i * L)) & 1u) {
                 const R n2 = col_norm2<RPL>(a[i]);
-                if (p == i) al = n2 * ((R)1 + da) * ((R)1 + da);
+                if (p == i) ca.n = n2 * ca.w() * ca.w();
             }
             if ((mb >> (i * L)) & 1u) {
                 const R n2 = col_norm2<RPL>(y[(i + r) % B]);
-                if (p == i) be = n2 * ((R)1 + db) * ((R)1 + db);
+                if (p == i) cy.n = n2 * cy.w() * cy.w();
             }
         }
     }
@@ -632,35 +714,29 @@ __device__ __forceinline__ unsigned round_pairs(entry_t<R> (&a)[B][RPL], entry_t
 }
 
 template <typename R, int RPL, int B, int r>
-__device__ __forceinline__ unsigned visit_rounds(entry_t<R> (&a)[B][RPL], entry_t<R> (&y)[B][RPL], R& al, R& da, int& fa,
-                                                 R& be, R& db, int& fb, Sweep<R>& sw, Coef<R>* tb, int lane) {
+__device__ __forceinline__ unsigned visit_rounds(entry_t<R> (&a)[B][RPL], entry_t<R> (&y)[B][RPL], Lane<R>& ca,
+                                                 Lane<R>& cy, Sweep<R>& sw, Coef<R>* tb, int lane) {
     if constexpr (r == B) {
         return 0u;
     } else {
-        unsigned m = round_pairs<R, RPL, B, r>(a, y, al, da, fa, be, db, fb, true, sw, tb, lane);
-        if constexpr (B > 1) {  // lane group p goes on to column (p + r + 1) mod B of y
-            constexpr int L = 32 / B;
-            const int src = (lane + L) & 31;
-            be = __shfl_sync(0xffffffffu, be, src);
-            db = __shfl_sync(0xffffffffu, db, src);
-            if constexpr (std::is_same<R, double>::value) fb = __shfl_sync(0xffffffffu, fb, src);
-        }
-        return m | visit_rounds<R, RPL, B, r + 1>(a, y, al, da, fa, be, db, fb, sw, tb, lane);
+        unsigned m = round_pairs<R, RPL, B, r>(a, y, ca, cy, sw, tb, lane);
+        if constexpr (B > 1) cy.move((lane + 32 / B) & 31);  // lane group p goes on to column (p + r + 1) mod B of y
+        return m | visit_rounds<R, RPL, B, r + 1>(a, y, ca, cy, sw, tb, lane);
     }
 }
 
-// Multiply the scales out: column i of a by 1 + (the da of lane group i).
+// Multiply the scales out: column i of a by the scale of lane group i.
 template <typename R, int RPL, int B>
-__device__ __forceinline__ void apply_scales(entry_t<R> (&a)[B][RPL], R& da) {
+__device__ __forceinline__ void apply_scales(entry_t<R> (&a)[B][RPL], Lane<R>& c) {
 #pragma unroll
-    for (int i = 0; i < B; ++i) col_scale<RPL>(a[i], __shfl_sync(0xffffffffu, da, i * (32 / B)));
-    da = 0;
+    for (int i = 0; i < B; ++i) col_scale<RPL>(a[i], __shfl_sync(0xffffffffu, c.d, i * (32 / B)));
+    c.d = (R)0;
+    c.i = 1;
 }
 
 // The pairs inside a group.
 template <typename R, int RPL, int B>
-__device__ __forceinline__ bool inner_pairs(entry_t<R> (&a)[B][RPL], R& al, R& da, int& fa, Sweep<R>& sw, Coef<R>* tb,
-                                            int lane) {
+__device__ __forceinline__ bool inner_pairs(entry_t<R> (&a)[B][RPL], Lane<R>& c, Sweep<R>& sw, Coef<R>* tb, int lane) {
     if constexpr (B == 1) {
         return false;
     } else {
@@ -684,11 +760,10 @@ __device__ __forceinline__ bool inner_pairs(entry_t<R> (&a)[B][RPL], R& al, R& d
                     z[1][q] = a[z1][q];
                 }
             }
-            const int sx = (ph == 0 ? x0 : x1) * L, sz = (ph == 0 ? z0 : z1) * L;
-            R ax = __shfl_sync(0xffffffffu, al, sx), az = __shfl_sync(0xffffffffu, al, sz);
-            R dx = __shfl_sync(0xffffffffu, da, sx), dz = __shfl_sync(0xffffffffu, da, sz);
-            int fx = __shfl_sync(0xffffffffu, fa, sx), fz = __shfl_sync(0xffffffffu, fa, sz);
-            const unsigned m = round_pairs<R, RPL, H, 0>(x, z, ax, dx, fx, az, dz, fz, true, sw, tb, lane);
+            Lane<R> cx = c, cz = c;
+            cx.move((ph == 0 ? x0 : x1) * L);
+            cz.move((ph == 0 ? z0 : z1) * L);
+            const unsigned m = round_pairs<R, RPL, H, 0>(x, z, cx, cz, sw, tb, lane);
             if (m) {
                 any |= m;
 #pragma unroll
@@ -703,14 +778,10 @@ __device__ __forceinline__ bool inner_pairs(entry_t<R> (&a)[B][RPL], R& al, R& d
                 // back to one lane group per column
                 const int p = lane / L;
                 const bool is_x = p == x0 || (H == 2 && p == x1);
-                const int pair = (p == x0 || p == z0) ? 0 : 1;
-                const int src = pair * LH;
-                const R bx = __shfl_sync(0xffffffffu, ax, src), bz = __shfl_sync(0xffffffffu, az, src);
-                const R ex = __shfl_sync(0xffffffffu, dx, src), ez = __shfl_sync(0xffffffffu, dz, src);
-                const int gx = __shfl_sync(0xffffffffu, fx, src), gz = __shfl_sync(0xffffffffu, fz, src);
-                al = is_x ? bx : bz;
-                da = is_x ? ex : ez;
-                fa = is_x ? gx : gz;
+                const int src = ((p == x0 || p == z0) ? 0 : 1) * LH;
+                cx.move(src);
+                cz.move(src);
+                c = is_x ? cx : cz;
             }
         };
         one(std::integral_constant<int, 0>{});
@@ -726,7 +797,6 @@ __device__ __forceinline__ bool inner_pairs(entry_t<R> (&a)[B][RPL], R& al, R& d
 constexpr int kMaxCols = 2 * PTEBD_CHI_LIMIT;  // 512
 constexpr int kMaxSlots = 32;
 constexpr int kMaxWarps = 16;
-constexpr double kScaleMax = 1.0 / 64;
 constexpr int kLag = 6;  // positions between a group's way back to W and the reuse of its slot
 
 // Tables of a CTA, ahead of the columns in shared memory.
@@ -796,7 +866,7 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
     // columns in shared memory start as zeros (rows beyond `rows` stay zero)
     for (int e = tid; e < (RES ? held + 1 : S * B + 1) * mpad; e += blockDim.x) cbuf[e] = cmake<C>(0, 0);
     for (int c = tid; c < cols; c += blockDim.x) {
-        T->scl[c] = 0;
+        T->scl[c] = (R)0;
         if constexpr (kSkip) T->flag[c] = 1;  // sweep 0 checks every pair
     }
     fence_async_smem();
@@ -862,6 +932,7 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
     const R tol = (R)(Eps<R>::k * sqrt((double)rows) * Eps<R>::u);
     Sweep<R> sw;
     sw.tol2 = tol * tol;
+    sw.tol2f = (float)sw.tol2;
     sw.big2 = (R)Eps<R>::early * sw.tol2;
     const bool polish = A.polish && Eps<R>::polish > 0.0;
     bool polishing = false;  // the last sweep, with the tighter threshold
@@ -985,6 +1056,19 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                 return fine;
             };
             const bool fetcher = !RES && warp == nwc - 1;
+            // column p of group g, from its tables
+            auto lane_of = [&](const Tables<R>* t, int g) {
+                const int pos = g * B + p;
+                Lane<R> c{(R)0, (R)0, (R)1, 0};
+                if (pos < cols) {
+                    c.n = t->pnrm[pos];
+                    c.d = t->pscl[pos];
+                    if constexpr (kSkip) {
+                        c.f = t->pflag[pos];
+                    }
+                }
+                return c;
+            };
             if (fetcher) {
                 if (lane == 0) { T->fetch_e = T->fetch_k = T->fetch_g = 0; T->fetch_slot = slot; }
                 __syncwarp();
@@ -1028,9 +1112,8 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
 #pragma unroll
                 for (int i = 0; i < B; ++i) col_load<RPL>(a[i], sm_col(I, i), lane);
                 const bool ip = I * B + p < cols;
-                R al = ip ? ti->pnrm[I * B + p] : (R)0, da = ip ? ti->pscl[I * B + p] : (R)0;
-                int fa = 0;
-                if constexpr (kSkip) fa = ip ? ti->pflag[I * B + p] : 0;
+                Lane<R> ca = lane_of(ti, I);
+                if constexpr (kSkip) ca.i = rcp_newton(ca.w());
                 bool changed = !RES && T->aux[I] != 0;
                 __syncwarp();
                 if (lane == 0) release(&ti->prog[I], I + 1);
@@ -1038,29 +1121,31 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                     if (lane == 0)
                         for (int q = 0; q < nwc; ++q) bulk_commit();
                 }
-                changed = inner_pairs<R, RPL, B>(a, al, da, fa, sw, tb, lane) || changed;
+                changed = inner_pairs<R, RPL, B>(a, ca, sw, tb, lane) || changed;
                 for (int J = I + 1; J < G; ++J) {
                     advance(1);
                     Tables<R>* const tj = home(J);
                     if (!ready(J, tj)) { ok = false; break; }
                     const bool jp = J * B + p < cols;
-                    R be = jp ? tj->pnrm[J * B + p] : (R)0, db = jp ? tj->pscl[J * B + p] : (R)0;
-                    int fb = 0;
-                    if constexpr (kSkip) fb = jp ? tj->pflag[J * B + p] : 0;
+                    Lane<R> cy = lane_of(tj, J);
                     bool store = last && T->aux[J] != 0;
-                    if (!kSkip || __any_sync(0xffffffffu, fa | fb)) {
+                    if (!kSkip || __any_sync(0xffffffffu, ca.f | cy.f)) {
+                        if constexpr (kSkip) {  // (the reciprocals, the I one's refreshed: it runs along)
+                            cy.i = rcp_newton(cy.w());
+                            ca.i = fma(ca.i, fma(-ca.w(), ca.i, 1.0), ca.i);
+                        }
                         entry_t<R> y[B][RPL];
 #pragma unroll
                         for (int i = 0; i < B; ++i) col_load<RPL>(y[i], sm_col(J, i), lane);
-                        if (visit_rounds<R, RPL, B, 0>(a, y, al, da, fa, be, db, fb, sw, tb, lane)) {
+                        if (visit_rounds<R, RPL, B, 0>(a, y, ca, cy, sw, tb, lane)) {
                             changed = true;
                             store = last;
-                            if (__any_sync(0xffffffffu, fabs(db) > (R)kScaleMax)) apply_scales<R, RPL, B>(y, db);
-                            if (__any_sync(0xffffffffu, fabs(da) > (R)kScaleMax)) apply_scales<R, RPL, B>(a, da);
+                            if (__any_sync(0xffffffffu, cy.far())) apply_scales<R, RPL, B>(y, cy);
+                            if (__any_sync(0xffffffffu, ca.far())) apply_scales<R, RPL, B>(a, ca);
                             if (jp && (lane & (L - 1)) == 0) {
-                                tj->pnrm[J * B + p] = be;
-                                tj->pscl[J * B + p] = db;
-                                if constexpr (kSkip) tj->pflag[J * B + p] = (unsigned char)fb;
+                                tj->pnrm[J * B + p] = cy.n;
+                                tj->pscl[J * B + p] = cy.d;
+                                if constexpr (kSkip) tj->pflag[J * B + p] = (unsigned char)cy.f;
                             }
 #pragma unroll
                             for (int i = 0; i < B; ++i)
@@ -1091,7 +1176,7 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                 }
                 if (!ok) break;
                 if (changed) {
-                    if (ip && (lane & (L - 1)) == 0) ti->pscl[I * B + p] = da;
+                    if (ip && (lane & (L - 1)) == 0) ti->pscl[I * B + p] = ca.d;
 #pragma unroll
                     for (int i = 0; i < B; ++i)
                         if (I * B + i < cols) {
@@ -1099,7 +1184,7 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                             else col_store<RPL>(a[i], W + (size_t)T->cperm[I * B + i] * ldw, lane, rows);
                         }
                     if constexpr (kSkip)
-                        if (ip && (lane & (L - 1)) == 0) ti->pflag[I * B + p] = (unsigned char)fa;
+                        if (ip && (lane & (L - 1)) == 0) ti->pflag[I * B + p] = (unsigned char)ca.f;
                 }
                 if (fetcher) pump(rel, true);  // rows shorter than the ring wait for all that was stored
                 advance(1);
