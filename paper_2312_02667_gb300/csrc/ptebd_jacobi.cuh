@@ -948,17 +948,21 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
     int sweep = 0;
     Coef<R>* tb = T->tb[warp];
 
+    // (one CTA streams columns of 12 and 16 rows a lane, however few)
+    const bool twos = RES && (!CL || (RPL < 12 && (cols + 1) * mpad * (int)sizeof(C) <= area));
     bool busy = true;        // a third of the pairs rotated in the last sweep
     bool last_tail = false;  // the polish sweep may leave pairs of dropped columns alone
     int run = 1;             // sweeps between two sorts
     for (sweep = 0; sweep < max_sweeps; sweep += run) {
-        // Resident columns: while a third of the pairs rotate, sweeps run into each other in twos,
-        // the second starting behind the first without a barrier, in the same order of columns.
-        // The pipeline of groups fills and drains once (3 G visits instead of 4 G for G groups and
-        // as many warps); later sweeps are sorted each, which saves more rotations than it costs.
-        // complex64 25 of 128 x 128 1.58 -> 1.47 ms.
+        // Columns that one CTA holds: while a third of the pairs rotate, sweeps run into each
+        // other in twos, the second starting behind the first without a barrier, in the same order
+        // of columns.  The pipeline of groups fills and drains once (3 G visits instead of 4 G for
+        // G groups and as many warps); later sweeps are sorted each, which saves more rotations
+        // than it costs.  complex64 25 of 128 x 128 1.58 -> 1.47 ms.  By size and not by where the
+        // columns are: what a cluster holds is streamed in a larger launch, and both have to give
+        // the same bits.
         // (Not a polish sweep: with GI < G the groups beyond never finish a sweep of their own.)
-        run = RES && !polishing && busy && sweep + 2 <= max_sweeps ? 2 : 1;
+        run = twos && !polishing && busy && sweep + 2 <= max_sweeps ? 2 : 1;
         norm_pass(sweep == 0);
         sync();
         if (sweep == 0) {
