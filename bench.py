@@ -63,7 +63,7 @@ def code_digest(text):
 
 
 def jacobi_traffic():
-    path = os.path.join(ROOT, "paper_2312_02667_gb300", "csrc", "ptebd_jacobi.cu")
+    path = os.path.join(ROOT, "paper_2312_02667_gb300", "csrc", "ptebd_jacobi.cuh")
     try:
         with open(path, encoding="utf-8") as f:
             digest = code_digest(f.read())
@@ -416,8 +416,8 @@ def run_ours(args, rank, world, local_rank):
             "traffic": jacobi_traffic() if args.precision == "mixed" and args.n_sites == 1024 and args.chi == 256 else None,
             "traffic_note": "bytes per launch, averaged over the three Jacobi launches of a step that runs every PtSU half-step "
                             "(gated 512x512 + two tSU passes on M^dag; ncu capture with --no-ptsu-shortcut --chunk-streams 1); "
-                            "the blocked Jacobi streams every matrix past its register-resident 16-column block "
-                            "nb(nb-1)/2 times per sweep, and 152 concurrent 2 MB matrices exceed L2",
+                            "for every n groups of columns that the n warps hold in registers, the later columns of the "
+                            "matrix are streamed past once per sweep, and 152 concurrent 2 MB matrices exceed L2",
             "algorithmic": "28 flop per column-pair-row visit x sweeps x n(n-1)/2 x m, counted on the device",
             "peak_source": peak_note,
             "svd_share_of_single_stream_step": svd_ms / sum(v[0] for v in kern.values()) if kern else None,

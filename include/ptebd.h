@@ -184,9 +184,9 @@ int ptebd_set_regauge_precision(ptebd_state* st, int32_t precision);
  * |a^H b| > 8 sqrt(rows) 2^-24 |a| |b| (or every rotation of a sweep was
  * small), which leaves the kept singular vectors orthogonal to about that
  * level; the truncated two-site state then carries a relative error of a few
- * 1e-5.  mode 1: the gated SVDs end with one more sweep at 2 sqrt(rows)
- * 2^-24, mode 2 (the default): the tSU SVDs as well, mode 3: the tSU SVDs
- * only, mode 0: none.  Measured on one saturated layer with PtSU (N = 256,
+ * 1e-5.  mode 1: the last sweeps of the gated SVDs, from when few pairs rotate,
+ * have the threshold sqrt(rows) 2^-24, mode 2 (the default): the tSU SVDs as well, mode 3: the tSU SVDs
+ * only, mode 0: none.  Measured with a threshold of 2 sqrt(rows) 2^-24 on one saturated layer with PtSU (N = 256,
  * chi = 256) against the FP64 path: 1 - F = 5.6e-7 (mode 0), 4.5e-7 (mode 1),
  * 4.7e-8 (mode 2) for 9% more time; at N = 1024, chi = 256: 3.2e-7 (mode
  * 2), 1.7e-6 (mode 3, 4% faster), 4.9e-6 (mode 0).  PTEBD_ERR_INVALID for
@@ -195,7 +195,7 @@ int ptebd_set_svd_polish(ptebd_state* st, int32_t mode);
 
 /* Tensor cores for a PTEBD_MIXED state (no counterpart in the paper: a
  * choice of arithmetic unit).  When chi_max rounded up (16 * 2^k) is at
- * least 64, enable = 1 (the default; any value other than 0 and 2): theta' =
+ * least 256 (smaller products always take the CUDA cores), enable = 1 (the default; any value other than 0 and 2): theta' =
  * U theta and the GEMM factor of the Gamma rebuild of gated bonds are formed by
  * tcgen05.mma kind::tf32 with FP32 accumulation in tensor memory, operands
  * split as hi + lo TF32 pairs and multiplied hi*hi + hi*lo + lo*hi (FP32
@@ -217,7 +217,8 @@ int ptebd_set_tensor_cores(ptebd_state* st, int32_t enable);
  * launch choice).  complex64: 16 (default), the warps and the shared memory of a
  * whole SM for each bond, or 8, at most 4 warps and half the shared memory;
  * complex128: always 8.  0 selects the default.  Results are bit-identical run to
- * run; the column pairs are met in the same order at either width.
+ * run at one width (a matrix that only the full shared memory holds takes its
+ * first sweeps in twos at width 16, and one by one at width 8).
  * PTEBD_ERR_INVALID for other widths. */
 int ptebd_set_jacobi_width(ptebd_state* st, int32_t nw);
 

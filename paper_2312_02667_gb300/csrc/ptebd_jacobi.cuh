@@ -35,7 +35,8 @@
 //
 // A pair (a, b) with |a^H b| > tol ||a|| ||b|| is rotated; the sweeps stop when
 // none was (or, on the complex64 path, when every rotation of a sweep was a
-// small one: Eps).  The squared column norms are recomputed at the start of every
+// small one: Eps).  Where one CTA can hold the columns, the first sweeps run in
+// twos without a sort and a barrier between (jacobi_body).  The squared column norms are recomputed at the start of every
 // sweep and tracked through the rotations in between; a norm that drops a lot
 // is recomputed from the rotated column.  On exit the columns are U S
 // (orthogonal, unsorted); their FP64 norms are the singular values.
@@ -196,8 +197,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
 // the columns are left orthogonal to about tol instead of below tol.
 // range_e: matrices whose largest entry is not in [2^-range_e, 2^range_e) are
 // rescaled before the sweeps (see the range guard in jacobi_body).
-// polish: the factor of a last sweep's tighter threshold (A.polish), run once
-// after the stopping rule has fired: it rotates every pair with
+// polish: the factor of the last sweeps' tighter threshold (A.polish), taken once
+// few pairs rotate (kPolishShare) or the stopping rule has fired: they rotate every pair with
 // |a^H b| > polish sqrt(rows) u |a| |b|, which leaves the columns orthogonal to
 // near the rounding of their storage (the truncated state depends on it: at 2 an
 // observable after a 12-layer chi = 64 circuit is 1.2e-6 off the FP64 one, at 1
