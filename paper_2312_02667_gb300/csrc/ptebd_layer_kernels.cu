@@ -130,24 +130,35 @@ __global__ void __launch_bounds__(256) k_theta(LayerArgs<R> a) {
 #pragma unroll
                 for (int q = 0; q < 2; ++q) acc[s][t][i][q] = cz<C>();
 
-    for (int k0 = 0; k0 < cm; k0 += 16) {
-        for (int e = threadIdx.x; e < 1024; e += 256) {
-            const int s = e >> 9, rem = e & 511, kk = rem >> 5, al = rem & 31;
-            const int alpha = a0 + al, beta = k0 + kk;
-            C v = cz<C>();
-            if (alpha < cl && beta < cm)
-                v = cscale(cconv<C>(G0[s * slice + (size_t)beta * chip + alpha]), sL[al] * sM[beta]);
-            xs[s][kk][al] = v;
-        }
-        for (int e = threadIdx.x; e < 1024; e += 256) {
+    // The 16 inner indices after those being multiplied are on their way from memory: a block
+    // waits for its loads otherwise, 2 blocks of 8 warps an SM cannot hide them (a step at
+    // N = 1024, chi = 256, its gated theta' on the tensor cores: 18.5 -> 12.7 ms of theta).
+    C nx[4], ny[4];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int e = threadIdx.x + 256 * i;
+            {
+                const int s = e >> 9, rem = e & 511, kk = rem >> 5, al = rem & 31;
+                const int alpha = a0 + al, beta = k0 + kk;
+                nx[i] = alpha < cl && beta < cm ? cconv<C>(G0[s * slice + (size_t)beta * chip + alpha]) : cz<C>();
+            }
             const int t = e >> 9, rem = e & 511, gg = rem >> 4, kk = rem & 15;
             const int gamma = g0 + gg, beta = k0 + kk;
-            C v = cz<C>();
-            if (gamma < cr && beta < cm)
-                v = cscale(cconv<C>(G1[t * slice + (size_t)gamma * chip + beta]), sR[gg]);
-            ys[t][kk][gg] = v;
+            ny[i] = gamma < cr && beta < cm ? cconv<C>(G1[t * slice + (size_t)gamma * chip + beta]) : cz<C>();
+        }
+    };
+    fetch(0);
+    for (int k0 = 0; k0 < cm; k0 += 16) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int e = threadIdx.x + 256 * i, rem = e & 511, kk = rem >> 5, al = rem & 31, beta = k0 + kk;
+            xs[e >> 9][kk][al] = beta < cm ? cscale(nx[i], sL[al] * sM[beta]) : cz<C>();
+            const int gg = rem >> 4;
+            ys[e >> 9][rem & 15][gg] = cscale(ny[i], sR[gg]);
         }
         __syncthreads();
+        if (k0 + 16 < cm) fetch(k0 + 16);
 #pragma unroll 4
         for (int kk = 0; kk < 16; ++kk) {
             C x[2][2], y[2][2];
