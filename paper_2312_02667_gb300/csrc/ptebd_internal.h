@@ -151,6 +151,9 @@ cudaError_t launch_add_partials(const double* partials, int k, double* totals, c
 
 // A layer may run as up to kMaxChunks bond chunks on concurrent streams.
 constexpr int kMaxChunks = 16;
+// complex64 rows x cols matrices (a.count of them at a.w), met by blocks of 16 columns
+cudaError_t jacobi_blocks_prepare();
+cudaError_t launch_jacobi_blocks(const LayerArgs<float>& a, int rows, int cols, cudaStream_t s);
 template <typename R> cudaError_t jacobi_prepare();   // raises the dynamic smem limit
 int jacobi_block_width(int precision, int requested);  // the NW a launch with a.nw = requested uses
 

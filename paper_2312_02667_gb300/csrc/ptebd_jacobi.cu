@@ -20,6 +20,7 @@ template <> cudaError_t jacobi_prepare<float>() {
     cudaError_t e = jac::prepare32<4>();
     if (e == cudaSuccess) e = jac::prepare32<8>();
     if (e == cudaSuccess) e = jac::prepare32<16>();
+    if (e == cudaSuccess) e = jacobi_blocks_prepare();
     return e;
 }
 

@@ -1,7 +1,8 @@
 // Batched SVD entry point: the layer's one-sided Jacobi SVD (the SVD step of
 // the TEBD procedure, Sec. II C of arXiv:2312.02667) on caller matrices.
 //   k_svd_load  : copy each input matrix into the workspace (the SVD rotates in place)
-//   k_jacobi    : the layer's kernel (ptebd_jacobi.cu)
+//   the Jacobi SVD: of complex64 matrices whose vectors are asked for by blocks of 16
+//     columns (ptebd_jacobi_blocks.cu), else by the layer's kernel (ptebd_jacobi.cu)
 //   k_svd_store : sort the FP64 column norms, write the singular values in
 //                 descending order and, when asked, the left singular vectors.
 #include <algorithm>
@@ -124,7 +125,12 @@ int run_svd(int batch, int rows, int cols, const void* a, int lda, double* sigma
     la.chip = ldw / 2;
     la.max_sweeps = 40;
     la.pass = 0;
-    if (launch_jacobi<R>(la, s) != cudaSuccess) return PTEBD_ERR_CUDA;
+    cudaError_t e = cudaSuccess;
+    if constexpr (std::is_same<R, float>::value)
+        e = u ? launch_jacobi_blocks(la, rows, cols, s) : launch_jacobi<R>(la, s);
+    else
+        e = launch_jacobi<R>(la, s);
+    if (e != cudaSuccess) return PTEBD_ERR_CUDA;
     k_svd_store<R><<<batch, 512, 0, s>>>(static_cast<const C*>(ws.w), ldw, ws.norms, rows, cols, sigma,
                                           static_cast<C*>(u), ldu);
     if (cudaGetLastError() != cudaSuccess) return PTEBD_ERR_CUDA;
