@@ -68,6 +68,7 @@
 #include <type_traits>
 
 #include "ptebd_internal.h"
+#include "ptebd_vote.h"
 
 namespace ptebd {
 namespace jac {
@@ -1106,20 +1107,21 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                 const bool big0 = sw.big;
                 const bool last = !RES && I == min(k0 + nw, GI) - 1;  // the last warp of the row
                 // Group g has met every I before this one (streaming, the first warp of a row: it
-                // has been fetched).  The same answer on every lane: they read one address in
-                // one instruction, and a wait that did not succeed at once ends in a vote.
+                // has been fetched), the same answer on every lane (warp_ready).
+                auto vote = [](bool x) -> bool { return __all_sync(0xffffffffu, x); };
                 auto ready = [&](int g, Tables<R>* tg) -> bool {
                     if (RES ? row == 0 : warp == 0) {
                         if constexpr (!RES)
-                            if (!mbar_try_wait(&T->full[slot], phase))
-                                return __all_sync(0xffffffffu, mbar_wait(&T->full[slot], phase, abort_flag));
+                            return warp_ready(mbar_try_wait(&T->full[slot], phase), vote,
+                                              [&] { return mbar_wait(&T->full[slot], phase, abort_flag); });
                         return true;
                     }
                     const bool test = wait_test && sweep == 0 && row == 1 && g == 1;
-                    if ((CL ? counter_acquire_cluster(&tg->prog[g]) : counter_acquire(&tg->prog[g])) >= base + I && !test)
-                        return true;
-                    return __all_sync(0xffffffffu, counter_wait<CL>(&tg->prog[g], test ? 0x7fffffff : base + I, abort_flag,
-                                                                    test ? (1ll << 20) : kWaitLimit));
+                    const int met = CL ? counter_acquire_cluster(&tg->prog[g]) : counter_acquire(&tg->prog[g]);
+                    return warp_ready(met >= base + I && !test, vote, [&] {
+                        return counter_wait<CL>(&tg->prog[g], test ? 0x7fffffff : base + I, abort_flag,
+                                                test ? (1ll << 20) : kWaitLimit);
+                    });
                 };
                 auto release = [&](int* c, int v) {
                     if constexpr (CL) counter_release_cluster(c, v); else counter_release(c, v);
@@ -1200,6 +1202,7 @@ __device__ __noinline__ void jacobi_body(const LayerArgs<R>& A, cx_t<R>* W, int 
                         }
                     }
                     if (lane == 0) release(&tj->prog[J], base + I + 1);
+                    __syncwarp();
                     if (fetcher) pump(rel, false);
                 }
                 if (!ok) break;
