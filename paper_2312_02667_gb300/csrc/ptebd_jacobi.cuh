@@ -63,10 +63,9 @@
 // abort flag, drains the CTA's own copies, latches DERR_TIMEOUT and returns.
 #pragma once
 #include <cmath>
-#include <map>
-#include <mutex>
 #include <type_traits>
 
+#include "ptebd_device.h"
 #include "ptebd_internal.h"
 #include "ptebd_vote.h"
 
@@ -1456,23 +1455,24 @@ template <typename K> cudaError_t clusters_at_once(K kernel, int threads, size_t
     return cudaSuccess;
 }
 struct MostClusters { int n[kMaxCluster + 1]; };
-// The same, found on first use (zeros where the kernel cannot be launched so).
-template <typename R>
-const MostClusters& most_clusters(void (*kernel)(LayerArgs<R>, int)) {
-    static std::mutex mu;
-    static std::map<const void*, MostClusters> found;
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = found.find(reinterpret_cast<const void*>(kernel));
-    if (it == found.end()) {
-        MostClusters m{};
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
-            clusters_at_once(kernel, 256, kSmemMax, m.n) != cudaSuccess) {
-            cudaGetLastError();
-            m = MostClusters{};
-        }
-        it = found.emplace(reinterpret_cast<const void*>(kernel), m).first;
-    }
-    return it->second;
+// The same on the current device, found on first use there (zeros, and no clusters, where
+// the query fails).
+template <typename R> MostClusters most_clusters(void (*kernel)(LayerArgs<R>, int)) {
+    static PerDevice<const void*, MostClusters> found;
+    int device = 0;
+    if (cudaGetDevice(&device) != cudaSuccess) return MostClusters{};
+    return found.get(device, reinterpret_cast<const void*>(kernel), [&](MostClusters* m) {
+        const cudaError_t e = clusters_at_once(kernel, 256, kSmemMax, m->n);
+        if (e != cudaSuccess) cudaGetLastError();
+        return (int)e;
+    });
+}
+// The dynamic shared memory of a kernel that runs in clusters, and their number.  The
+// attribute belongs to the device's context: set on every call.
+template <typename R> cudaError_t prepare_clusters(void (*kernel)(LayerArgs<R>, int)) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+    if (e == cudaSuccess) most_clusters(kernel);
+    return e;
 }
 // CTAs for each of `bonds` matrices in flight together: as many as still run all at once.
 inline int cluster_for(int bonds, const int (&most)[kMaxCluster + 1]) {

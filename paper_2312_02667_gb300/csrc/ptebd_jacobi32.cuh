@@ -57,7 +57,8 @@ __global__ void __launch_bounds__(256, 1) k_jacobi_cluster(LayerArgs<float> A, i
 }
 
 template <int MAXRPL> cudaError_t prepare32() {
-    most_clusters(k_jacobi_cluster<MAXRPL>);
+    const cudaError_t e = prepare_clusters(k_jacobi_cluster<MAXRPL>);
+    if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(k_jacobi<MAXRPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
 }
 

@@ -42,7 +42,8 @@ __global__ void __launch_bounds__(256, 1) k_jacobi64(LayerArgs<double> A, int ar
 }
 
 template <int MAXRPL> cudaError_t prepare64() {
-    most_clusters(k_jacobi64<MAXRPL, true>);
+    const cudaError_t e = prepare_clusters(k_jacobi64<MAXRPL, true>);
+    if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(k_jacobi64<MAXRPL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
 }
 

@@ -23,3 +23,7 @@ def run_native(name, tmp_path):
 
 def test_a_warps_answer_is_the_same_on_every_lane(tmp_path):
     run_native("vote", tmp_path)
+
+
+def test_what_belongs_to_a_device(tmp_path):
+    run_native("device", tmp_path)
