@@ -19,6 +19,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "ptebd_device.h"
 #include "ptebd_internal.h"
 
 using namespace ptebd;
@@ -31,7 +32,7 @@ struct ptebd_state {
     size_t ws_bytes = 0;
     int slots = 0;
     cudaStream_t stream = nullptr;
-    int device = 0;
+    int device = 0;         // of the stream
     int layers = 0;
     std::string last_error;
     // per-kernel CUDA-event timing
@@ -662,6 +663,11 @@ int sync_and_check(ptebd_state* st) {
     return check_device_errors(st);
 }
 
+struct Cuda {
+    int get(int* d) { return (int)cudaGetDevice(d); }
+    int set(int d) { return (int)cudaSetDevice(d); }
+};
+
 // Small reads of the state.  One kernel gathers the pieces and the error word into
 // pinned host memory and one synchronisation brings them, where a copy and a
 // synchronisation each took 39 us for the three of a Schmidt spectrum (reading
@@ -694,6 +700,9 @@ int read_state(ptebd_state* st, std::initializer_list<Piece> pieces, const char*
         p.src[n] = static_cast<const uint32_t*>(x.src);
         p.words[n++] = (uint32_t)(x.bytes / 4);
     }
+    // a launch wants the stream's device to be current; a program may have another one
+    const OnDevice<Cuda> here(st->device);
+    if (here.error()) return set_err(st, PTEBD_ERR_CUDA, "device %d cannot be made current", st->device);
     k_read<<<1, 256, 0, st->stream>>>(p, at<uint32_t>(st->mem, st->L.off_err), reinterpret_cast<uint32_t*>(st->host));
     CUDA_TRY(st, cudaGetLastError());
     CUDA_TRY(st, cudaStreamSynchronize(st->stream));
@@ -1019,7 +1028,7 @@ int ptebd_create(const ptebd_config* cfg, void* state_mem, size_t state_bytes, v
     st->ws_bytes = workspace_bytes;
     st->slots = slots;
     st->stream = static_cast<cudaStream_t>(stream);
-    cudaGetDevice(&st->device);
+    if (cudaStreamGetDevice(st->stream, &st->device) != cudaSuccess) cudaGetDevice(&st->device);
     if (cudaHostAlloc(reinterpret_cast<void**>(&st->host), host_bytes(L), cudaHostAllocMapped) != cudaSuccess) {
         cudaGetLastError();
         st->host = nullptr;

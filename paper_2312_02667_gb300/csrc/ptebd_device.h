@@ -25,4 +25,25 @@ public:
     }
 };
 
+// `device` is the current one while this lives, then the one before again.  Api: int get(int*)
+// and int set(int), the runtime's calls.
+template <typename Api> class OnDevice {
+    Api api_;
+    int before_ = 0, error_;
+    bool changed_ = false;
+
+public:
+    OnDevice(int device, Api api = Api()) : api_(api), error_(api_.get(&before_)) {
+        if (error_ || before_ == device) return;
+        error_ = api_.set(device);
+        changed_ = !error_;
+    }
+    ~OnDevice() {
+        if (changed_) api_.set(before_);
+    }
+    OnDevice(const OnDevice&) = delete;
+    OnDevice& operator=(const OnDevice&) = delete;
+    int error() const { return error_; }
+};
+
 }  // namespace ptebd

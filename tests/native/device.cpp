@@ -1,5 +1,6 @@
 // PerDevice: a value of one device is not another's, a search that failed is made again, and
 // a value found is not searched for twice, by any number of threads.
+// OnDevice: the device is current inside, and the one before is afterwards.
 #include <atomic>
 #include <cstdio>
 #include <thread>
@@ -9,7 +10,36 @@
 
 #define CHECK(x) do { if (!(x)) { std::printf("line %d: %s\n", __LINE__, #x); return 1; } } while (0)
 
+struct Fake {
+    int* current;
+    int* sets;
+    int refuse;  // a device that cannot be made current
+    int get(int* d) { *d = *current; return 0; }
+    int set(int d) { ++*sets; if (d == refuse) return 101; *current = d; return 0; }
+};
+
+int on_device() {
+    int current = 0, sets = 0;
+    {
+        ptebd::OnDevice<Fake> here(0, Fake{&current, &sets, -1});
+        CHECK(here.error() == 0 && current == 0);
+    }
+    CHECK(sets == 0);  // (the usual case: nothing to do)
+    {
+        ptebd::OnDevice<Fake> there(1, Fake{&current, &sets, -1});
+        CHECK(there.error() == 0 && current == 1);
+    }
+    CHECK(current == 0 && sets == 2);
+    {
+        ptebd::OnDevice<Fake> there(3, Fake{&current, &sets, 3});
+        CHECK(there.error() == 101 && current == 0);
+    }
+    CHECK(current == 0 && sets == 3);
+    return 0;
+}
+
 int main() {
+    if (on_device()) return 1;
     ptebd::PerDevice<const void*, int> counts;
     int key_a = 0, key_b = 0, searches = 0;
     auto finds = [&](int v) { return [&searches, v](int* out) { ++searches; *out = v; return 0; }; };
