@@ -54,6 +54,7 @@ struct ptebd_state {
     int tensor_cores = 1;   // complex64 theta' on the tensor cores (ptebd_set_tensor_cores)
     int polish = 2;         // complex64 Jacobi polish sweep: 0 none, 1 gated SVDs, 2 gated and tSU, 3 tSU
     char* host = nullptr;   // pinned, mapped: where small reads of the state land (owned)
+    std::mutex read_mu;     // one read at a time has it
     cudaStream_t body_stream = nullptr;  // captures the bodies of the FP64 pass's IF nodes (owned)
     // set once a device error says that a CTA returned with its own bulk copies still in
     // flight (DERR_DRAIN): the state and its workspace can no longer be trusted, and
@@ -672,7 +673,7 @@ struct Cuda {
 // pinned host memory and one synchronisation brings them, where a copy and a
 // synchronisation each took 39 us for the three of a Schmidt spectrum (reading
 // all of them took as long as the layers of a 128-site, chi = 64 step).
-struct Piece { const void* src; size_t bytes; };  // bytes a multiple of 4, src 4-byte aligned
+struct Piece { const void* src; size_t bytes; void* dst; };  // bytes a multiple of 4, src 4-byte aligned; dst may be null
 struct Pieces { const uint32_t* src[4]; uint32_t words[4]; };
 constexpr size_t kHostHead = 16;  // the error word, ahead of the pieces
 
@@ -690,9 +691,10 @@ __global__ void __launch_bounds__(256) k_read(Pieces p, const uint32_t* err, uin
     }
 }
 
-// The pieces, one behind the other, at *data (valid until the next read); `check`: a
-// latched device error is reported (and cleared) instead.
-int read_state(ptebd_state* st, std::initializer_list<Piece> pieces, const char** data, bool check = true) {
+// The pieces, to their places on the host; `check`: a latched device error is reported (and
+// cleared) instead.  Any number of threads may read a state: the buffer is one read's until
+// its pieces have been copied out.
+int read_state(ptebd_state* st, std::initializer_list<Piece> pieces, bool check = true) {
     if (check && st->poisoned) return refuse_poisoned(st);
     Pieces p{};
     int n = 0;
@@ -700,6 +702,7 @@ int read_state(ptebd_state* st, std::initializer_list<Piece> pieces, const char*
         p.src[n] = static_cast<const uint32_t*>(x.src);
         p.words[n++] = (uint32_t)(x.bytes / 4);
     }
+    const std::lock_guard<std::mutex> lock(st->read_mu);
     // a launch wants the stream's device to be current; a program may have another one
     const OnDevice<Cuda> here(st->device);
     if (here.error()) return set_err(st, PTEBD_ERR_CUDA, "device %d cannot be made current", st->device);
@@ -708,16 +711,19 @@ int read_state(ptebd_state* st, std::initializer_list<Piece> pieces, const char*
     CUDA_TRY(st, cudaStreamSynchronize(st->stream));
     uint32_t err;
     std::memcpy(&err, st->host, sizeof err);
-    *data = st->host + kHostHead;
-    return check && err ? check_device_errors(st) : PTEBD_OK;
+    if (check && err) return check_device_errors(st);
+    const char* d = st->host + kHostHead;
+    for (const Piece& x : pieces) {
+        if (x.dst) std::memcpy(x.dst, d, x.bytes);
+        d += x.bytes;
+    }
+    return PTEBD_OK;
 }
 
 // Every bond dimension (n_sites + 1 of them), after the errors of the work before.
 std::vector<int32_t> host_chi(ptebd_state* st, int* rc, bool check = true) {
     std::vector<int32_t> chi((size_t)st->L.n_sites + 1);
-    const char* d;
-    *rc = read_state(st, {{at<int32_t>(st->mem, st->L.off_chi), chi.size() * sizeof(int32_t)}}, &d, check);
-    if (!*rc) std::memcpy(chi.data(), d, chi.size() * sizeof(int32_t));
+    *rc = read_state(st, {{at<int32_t>(st->mem, st->L.off_chi), chi.size() * sizeof(int32_t), chi.data()}}, check);
     return chi;
 }
 
@@ -1339,13 +1345,12 @@ int ptebd_get_chi(ptebd_state* st, int32_t* chi_out) {
 int ptebd_get_lambda(ptebd_state* st, int32_t bond, double* out, int32_t* k) {
     if (!st || !out) return set_err(st, PTEBD_ERR_INVALID, "null argument");
     if (bond < 0 || bond > st->L.n_sites - 2) return set_err(st, PTEBD_ERR_INVALID, "bond out of range");
-    const char* d;
-    const size_t row = (size_t)st->L.chip * sizeof(double);
-    const int rc = read_state(st, {{lam_ptr(st, bond), row}, {at<int32_t>(st->mem, st->L.off_chi) + bond + 1, 4}}, &d);
-    if (rc) return rc;
+    std::vector<double> row(st->L.chip);
     int32_t kk;
-    std::memcpy(&kk, d + row, sizeof kk);
-    std::memcpy(out, d, (size_t)kk * sizeof(double));
+    const int rc = read_state(st, {{lam_ptr(st, bond), row.size() * sizeof(double), row.data()},
+                                   {at<int32_t>(st->mem, st->L.off_chi) + bond + 1, sizeof kk, &kk}});
+    if (rc) return rc;
+    std::memcpy(out, row.data(), (size_t)kk * sizeof(double));
     if (k) *k = kk;
     return PTEBD_OK;
 }
@@ -1426,11 +1431,9 @@ int ptebd_set_site(ptebd_state* st, int32_t site, int32_t chi_l, int32_t chi_r, 
 
 int ptebd_trunc_error(ptebd_state* st, double* eps_total, double* log_nu_total) {
     if (!st) return PTEBD_ERR_INVALID;
-    const char* d;
-    const int rc = read_state(st, {{at<double>(st->mem, st->L.off_totals), 2 * sizeof(double)}}, &d);
-    if (rc) return rc;
     double t[2];
-    std::memcpy(t, d, sizeof t);
+    const int rc = read_state(st, {{at<double>(st->mem, st->L.off_totals), sizeof t, t}});
+    if (rc) return rc;
     if (eps_total) *eps_total = t[0];
     if (log_nu_total) *log_nu_total = t[1];
     return PTEBD_OK;
@@ -1439,15 +1442,9 @@ int ptebd_trunc_error(ptebd_state* st, double* eps_total, double* log_nu_total) 
 int ptebd_bond_stats(ptebd_state* st, double* eps, double* nu, int32_t* rank_in) {
     if (!st) return PTEBD_ERR_INVALID;
     const size_t nb = (size_t)st->L.n_sites - 1;
-    const char* d;
-    const int rc = read_state(st, {{at<double>(st->mem, st->L.off_bond_eps), nb * sizeof(double)},
-                                   {at<double>(st->mem, st->L.off_bond_nu), nb * sizeof(double)},
-                                   {at<int32_t>(st->mem, st->L.off_bond_rank), nb * sizeof(int32_t)}}, &d);
-    if (rc) return rc;
-    if (eps) std::memcpy(eps, d, nb * sizeof(double));
-    if (nu) std::memcpy(nu, d + nb * sizeof(double), nb * sizeof(double));
-    if (rank_in) std::memcpy(rank_in, d + 2 * nb * sizeof(double), nb * sizeof(int32_t));
-    return PTEBD_OK;
+    return read_state(st, {{at<double>(st->mem, st->L.off_bond_eps), nb * sizeof(double), eps},
+                           {at<double>(st->mem, st->L.off_bond_nu), nb * sizeof(double), nu},
+                           {at<int32_t>(st->mem, st->L.off_bond_rank), nb * sizeof(int32_t), rank_in}});
 }
 
 int ptebd_work_counters(ptebd_state* st, uint64_t* out, int32_t n) {
@@ -1716,10 +1713,8 @@ int ptebd_sample(ptebd_state* st, int32_t n_samples, const double* uniforms, int
 int ptebd_svd_sweeps(ptebd_state* st, int32_t* sweeps, int32_t* layers) {
     if (!st) return PTEBD_ERR_INVALID;
     const size_t nb = (size_t)st->L.n_sites - 1;
-    const char* d;
-    const int rc = read_state(st, {{at<int32_t>(st->mem, st->L.off_bond_sweeps), nb * sizeof(int32_t)}}, &d);
+    const int rc = read_state(st, {{at<int32_t>(st->mem, st->L.off_bond_sweeps), nb * sizeof(int32_t), sweeps}});
     if (rc) return rc;
-    if (sweeps) std::memcpy(sweeps, d, nb * sizeof(int32_t));
     if (layers) *layers = st->layers;
     return PTEBD_OK;
 }
