@@ -24,6 +24,16 @@
 
 using namespace ptebd;
 
+namespace {
+// While this lives, this thread may make calls that a stream capture, of its own or of another
+// thread, would forbid: states come and go whatever else is being captured.
+struct DuringCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    DuringCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~DuringCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+}  // namespace
+
 struct ptebd_state {
     ptebd_config cfg;
     Layout L;
@@ -66,7 +76,10 @@ struct ptebd_state {
         if (fork_ev) cudaEventDestroy(fork_ev);
         for (cudaStream_t x : aux) cudaStreamDestroy(x);
         if (body_stream) cudaStreamDestroy(body_stream);
-        if (host) cudaFreeHost(host);
+        if (host) {
+            const DuringCapture any;
+            cudaFreeHost(host);
+        }
     }
 };
 
@@ -1035,9 +1048,14 @@ int ptebd_create(const ptebd_config* cfg, void* state_mem, size_t state_bytes, v
     st->slots = slots;
     st->stream = static_cast<cudaStream_t>(stream);
     if (cudaStreamGetDevice(st->stream, &st->device) != cudaSuccess) cudaGetDevice(&st->device);
-    if (cudaHostAlloc(reinterpret_cast<void**>(&st->host), host_bytes(L), cudaHostAllocMapped) != cudaSuccess) {
-        cudaGetLastError();
-        st->host = nullptr;
+    {
+        const DuringCapture any;
+        if (cudaHostAlloc(reinterpret_cast<void**>(&st->host), host_bytes(L), cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();
+            st->host = nullptr;
+        }
+    }
+    if (!st->host) {
         delete st;
         return PTEBD_ERR_MEMORY;
     }
