@@ -37,20 +37,17 @@ UNIT = "bond-SVDs/s"
 SM_COUNT = 152
 
 # DRAM bytes (read + write) per k_jacobi launch, from one ncu capture of this
-# workload on one stream (--chunk-streams 1, the launches the roofline's
-# `achieved` is timed on; dram__bytes_read.sum + dram__bytes_write.sum of the
-# three Jacobi launches of one step, the gated SVDs and the two tSU passes on
-# M^dag: 291.2, 39.3, 28.9 GB at the first key, 315.8, 45.5, 35.3 GB at the
-# second, 315.7, 45.5, 35.3 GB at the third and 315.8, 45.5, 35.3 GB at the
-# fourth; averaged per launch), keyed by the SHA-256 of
-# the kernel source it was taken on, with comments and blank lines removed (a
-# comment edit leaves the key alone).  Any other code reports null: the
-# counters no longer describe the kernel.
+# workload on one stream (--chunk-streams 1 --no-ptsu-shortcut, the launches the
+# roofline's `achieved` is timed on; dram__bytes_read.sum + dram__bytes_write.sum of
+# the three Jacobi launches of one step, the gated SVDs and the two tSU passes on
+# M^dag; averaged per launch), keyed by the SHA-256 of the kernel's sources (the
+# sweeps, the warps of a class and the dispatch) with comments and blank lines
+# removed, so that a comment edit leaves the key alone.  Any other code reports null:
+# the counters no longer describe the kernel.
+JACOBI_SOURCES = ("ptebd_jacobi.cuh", "ptebd_jacobi32.cuh", "ptebd_jacobi.cu")
 JACOBI_TRAFFIC = {
-    "a673d11c5d5a93dc1bb29eacc0981c712ff478a81a49b8f0917de1ae980a5fa0": 359.46e9 / 3,
-    "67f5d33a0c769e2e0fea0fd8d30e312096ce4418525e18a236e430e26c66bc0b": 396.6e9 / 3,
-    "a9c859b525d94476efa21326b5bbd6f6759842cca47e2da411c8f315a9ccf676": 396.57e9 / 3,
-    "5491b7d858d3e01f7faed505b83a18a716618e41f84acfa5cb01c875475892d9": 396.59e9 / 3,
+    # 162.2, 19.2 and 16.2 GB
+    "a86964fc48df961004cb1bf02b82ba254ac80edd455425293faac20f89cb9626": 197.63e9 / 3,
 }
 
 
@@ -62,14 +59,19 @@ def code_digest(text):
     return hashlib.sha256("\n".join(ln for ln in lines if ln.strip()).encode()).hexdigest()
 
 
+def jacobi_digest():
+    text = ""
+    for name in JACOBI_SOURCES:
+        with open(os.path.join(ROOT, "paper_2312_02667_gb300", "csrc", name), encoding="utf-8") as f:
+            text += f.read() + "\n"
+    return code_digest(text)
+
+
 def jacobi_traffic():
-    path = os.path.join(ROOT, "paper_2312_02667_gb300", "csrc", "ptebd_jacobi.cuh")
     try:
-        with open(path, encoding="utf-8") as f:
-            digest = code_digest(f.read())
+        return JACOBI_TRAFFIC.get(jacobi_digest())
     except OSError:
         return None
-    return JACOBI_TRAFFIC.get(digest)
 
 
 def parse():
@@ -108,7 +110,7 @@ def parse():
     p.add_argument("--jacobi-width", type=int, default=0, choices=[0, 8, 16],
                    help="complex64 Jacobi block width (0: the library's choice)")
     p.add_argument("--jacobi-pairs", type=int, default=0, choices=[0, 1, 2],
-                   help="complex64 Jacobi I columns per warp at width 16 (0: the library's choice)")
+                   help="accepted, without effect: a warp holds a whole group of columns")
     p.add_argument("--resolve", type=float, default=-1.0,
                    help="mixed: the level below which complex64 singular values are resolved in FP64 (-1: default)")
     p.add_argument("--qft", action="store_true",
@@ -392,7 +394,6 @@ def run_ours(args, rank, world, local_rank):
         "jacobi_width": args.jacobi_width or "library choice",
         "tensor_cores": "off" if args.no_tensor_cores else ("gated and tSU" if args.tsu_tensor_cores else "gated stages"),
         "svd_polish": args.svd_polish if args.svd_polish >= 0 else "library choice",
-        "jacobi_columns_per_warp": args.jacobi_pairs or "library choice",
         "kernels_ms_per_step": {k: v[0] / diag_layers for k, v in kern.items()},
         "kernels_note": ("per-kernel CUDA-event times from a separate pass of the next two layers on one stream "
                          "(events around every launch serialise the chunks); the timed steps run the chunks "
@@ -708,9 +709,8 @@ def serving_bench(args):
         choices[kk] = st.autotune(gates, parity)
     tune_s = time.perf_counter() - t0
     for i, st in enumerate(states):
-        nw, chunks, _, _, pairs = choices[key(i)]
+        nw, chunks = choices[key(i)][:2]
         st.set_jacobi_width(nw)
-        st.set_jacobi_pairs(pairs)
         st.set_chunk_streams(chunks)
     first_t, wall_t, dev_t, _ = run_pass()
     for st in states:
@@ -721,7 +721,7 @@ def serving_bench(args):
             "untuned": {"value": gated / wall_u, "wall_s": wall_u, "device_s": dev_u, "first_pass_s": first_u},
             "tuned": {"value": gated / wall_t, "wall_s": wall_t, "device_s": dev_t, "first_pass_s": first_t,
                       "tuning_s": tune_s,
-                      "choices": {f"chi{a}_nbits{b}": {"jacobi_width": c[0], "chunks": c[1], "columns_per_warp": c[4]}
+                      "choices": {f"chi{a}_nbits{b}": {"jacobi_width": c[0], "chunks": c[1]}
                                   for (a, b), c in choices.items()}},
             "circuit_layers_per_s": float(ds.sum()) / wall_t, "batch_layers_per_s": len(layers) / wall_t,
             "gated_bond_updates": gated, "fp64_resolved_bonds": resolved,
