@@ -398,7 +398,7 @@ int ptebd_batch_apply_layer(ptebd_batch* b, const double* const* gates, const in
  *    complex64, after a sweep whose rotated pairs all had cos^2 < 256 tol^2
  *    (the sweep after such a sweep was measured to find no pair above
  *    1.04 tol^2).  What is left within tol depends on the order in which the
- *    columns meet, 1e-4 of U S^-1 (U^H A) at 300 rows: complex64 vectors
+ *    columns meet, about 1e-4 of U S^-1 (U^H A) at 300 rows: complex64 vectors
  *    always come from blocks of 16 columns in row-cyclic order, while calls
  *    for singular values alone run the layers' kernel, 1.5 to 4 times faster.
  * workspace: device, 256-byte aligned, at least ptebd_svd_workspace_bytes.

@@ -12,14 +12,14 @@
 // operator's entries over their trace, so numerator and denominator share
 // everything.
 //
-//   k_zmm     : a batch of up to four complex products, k in one or two segments,
+//   k_zmm     : a batch of up to eight complex products, k in one or two segments,
 //               rows and columns scaled, with the largest modulus of the result
 //               gathered so that the next step can take a power of two out;
 //   k_overlaps: sums of conj(P) Q;
 //   k_sample_pick.
 //
 // What bounds it: the FP64 pipe (2 fused multiply-adds per SM and cycle: a 64 x 64 x
-// 64 complex product is 3.5 us of the whole chip) and, at small bond dimensions, the
+// 64 complex product is 1.7 us of the whole chip) and, at small bond dimensions, the
 // latency of a launch.  Hence 4 x 8 output tiles of 128 threads: chi = 64 gives 256
 // tiles a side (32 x 32 tiles of 256 threads kept 4 of 152 SMs busy at 65 us a
 // product; 64 threads leave two of an SM's four FP64 units idle), and two launches

@@ -106,9 +106,9 @@ struct LayerArgs {
     int wait_test;    // test of the bounded waits: one hand-off wait per CTA targets a count nothing
                       // reaches, with a short limit, so the CTA aborts and latches DERR_TIMEOUT
     int nw;           // Jacobi block width requested (complex64: 8 halves a CTA's warps and shared memory)
-    int tensor_cores; // complex64 on the tensor cores (tcgen05, 3xTF32) when chip >= 128: 1 theta' and
+    int tensor_cores; // complex64 on the tensor cores (tcgen05, 3xTF32) when chip >= 256: 1 theta' and
                       // the Gamma GEMM of gated stages, 2 the tSU steps as well
-    int polish;       // complex64 Jacobi: one last sweep at the tighter threshold (see Eps::polish)
+    int polish;       // complex64 Jacobi: the last sweeps at the tighter threshold (see Eps::polish)
     int mode;         // 0: gated bond; 1: tSU through the rank-chi_b factorisation
     int pass;         // Jacobi: 0 = rows/cols from dims, 1 = the X factor (2 chi_{b-1} x chi_b)
     double* bond_eps; double* bond_nu; int32_t* bond_rank; int32_t* bond_sweeps;

@@ -44,9 +44,9 @@
 // What bounds it: on complex64 the latency of a round's chain (dot products,
 // shuffles, the rotation, coefficients through shared memory), two or three warps
 // per scheduler; on complex128 the FP64 pipe.  Against one column per warp and a
-// rotation worked out by every lane of every pair (the kernel before this one):
-// 152 Ginibre matrices, complex64 128 x 128 3.81 -> 2.06 ms, 256 x 256 17.3 -> 9.0,
-// 512 x 512 95 -> 76; complex128, 64 of 128 x 128 98.6 -> 42.8 ms.  Why the groups go
+// rotation worked out by every lane of every pair (the kernel before this one, which
+// ptebd_jacobi_blocks.cu keeps): 152 Ginibre matrices, complex64 128 x 128 3.48 -> 1.89 ms,
+// 256 x 256 16.8 -> 8.6, 512 x 512 89 -> 67; complex128 128 x 128 99 -> 40.  Why the groups go
 // in row-cyclic order: a tournament over all groups would keep every warp busy
 // but takes 13 to 16 sweeps where this order takes 10 or 11.
 //
@@ -54,8 +54,8 @@
 // columns lie in the shared memory of all of them, the warps of all of them make
 // one row of I groups, and counters, norms and scales are read through distributed
 // shared memory.  The arithmetic and its order are the same, so the result does
-// not depend on how a matrix was spread.  10 complex128 256 x 256: 313 -> 71 ms
-// (8 CTAs each), 64 of 128 x 128: 41 -> 28 (2 each); complex64 37 of 200 x 200
+// not depend on how a matrix was spread.  10 complex128 256 x 256: 313 -> 68 ms
+// (8 CTAs each), 64 of 128 x 128: 41 -> 27 (2 each); complex64 37 of 200 x 200
 // 5.6 -> 3.6 (3 or 4 each).  Each launch takes the largest cluster at which all its
 // matrices still run at once (cluster_for).
 //
@@ -255,11 +255,6 @@ __device__ __forceinline__ float2 upk2(unsigned long long v) {
 __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
     unsigned long long d;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
 
@@ -791,9 +786,14 @@ __device__ __forceinline__ bool inner_pairs(entry_t<R> (&a)[B][RPL], Lane<R>& c,
 constexpr int kMaxCols = 2 * PTEBD_CHI_LIMIT;  // 512
 constexpr int kMaxSlots = 32;
 constexpr int kMaxWarps = 16;
-// Of cols (cols - 1): a sweep that rotates more lets the next two run into each other.
+// Of cols (cols - 1): a sweep that rotates more lets the next two run into each other.  Flat
+// around 0.3 of the pairs: at 0.15, 0.3, 0.5 and never, a step of N = 16, chi = 16 takes 1.150,
+// 1.146, 1.153 and 1.206 ms, of N = 128, chi = 64 7.59, 7.56, 7.55 and 7.83 (in FP64 82.4, 82.5,
+// 82.4 and 84.8), a 12-layer circuit of N = 50, chi = 64 13.4, 13.5, 13.6 and 14.7.
 constexpr float kBusyShare = 0.3f / 2;
 // Of cols (cols - 1): a sweep that rotates fewer pairs hands the next the polish threshold.
+// At none, 0.05, 0.15 and 0.3 of the pairs the same steps take 1.163, 1.162, 1.146 and 1.148,
+// and 7.72, 7.63, 7.56 and 7.51 ms, one of N = 75, chi = 100 8.69, 8.76, 8.66 and 8.70.
 constexpr float kPolishShare = 0.15f / 2;
 constexpr int kLag = 6;  // positions between a group's way back to W and the reuse of its slot
 
@@ -817,7 +817,7 @@ template <typename R> struct Tables {
     int fetch_e, fetch_k, fetch_g, fetch_slot;  // streaming: the next position to fetch, its row, group and slot
 };
 
-// Smallest power of two >= 1 + the table size, so that the columns start 128-byte aligned.
+// The tables, rounded up to 128 bytes, so that the columns start aligned.
 template <typename R> constexpr size_t table_bytes() { return (sizeof(Tables<R>) + 127) / 128 * 128; }
 
 // Dynamic shared memory: the tables and `column_area` bytes of columns.

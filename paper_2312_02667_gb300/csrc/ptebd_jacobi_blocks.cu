@@ -3,10 +3,10 @@
 //
 // The sweeps stop with the columns orthogonal to 8 sqrt(rows) 2^-24, and what is left
 // below that depends on the order in which the pairs met: the isometry U S^-1 (U^H A)
-// of a 300 x 240 Ginibre matrix lies 1.3e-4 off the exact one, in another direction for
+// of a 300 x 240 Ginibre matrix lies 1.2e-4 off the exact one, in another direction for
 // every order.  Callers hold vectors of the order below, so these keep it, where the
 // pipeline of column groups (ptebd_jacobi.cuh, which takes the layers and the calls for
-// singular values alone) would move them by 1.7e-4.
+// singular values alone) would move them by as much.
 //
 // One CTA of 16 warps a matrix; the columns stay in global memory / L2.  Blocks of 16
 // columns, by decreasing column norm (re-sorted at the start of every sweep), meet in
@@ -55,6 +55,11 @@ __device__ __forceinline__ void counter_release_add(int* p) {
 }
 __device__ __forceinline__ void bulk_wait_read_all() {
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
 }
 __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
     unsigned long long d;
