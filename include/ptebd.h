@@ -400,7 +400,7 @@ int ptebd_batch_apply_layer(ptebd_batch* b, const double* const* gates, const in
  *    1.04 tol^2).  What is left within tol depends on the order in which the
  *    columns meet, about 1e-4 of U S^-1 (U^H A) at 300 rows: complex64 vectors
  *    always come from blocks of 16 columns in row-cyclic order, while calls
- *    for singular values alone run the layers' kernel, 1.5 to 4 times faster.
+ *    for singular values alone run the layers' kernel, 1.3 to 4 times faster.
  * workspace: device, 256-byte aligned, at least ptebd_svd_workspace_bytes.
  * The input is not modified.  Runs on `stream` (cudaStream_t).  check != 0
  * synchronises the stream and reports device errors (sweep limit, non-finite

@@ -23,8 +23,7 @@
 // the unit roundoff.
 //
 // What bounds it: the latency of a pair's chain, one pair a warp.  152 matrices of
-// 64 x 50, 128 x 100, 256 x 200 and 512 x 400: 0.85, 2.76, 11.2 and 62.3 ms (values alone in
-// the pipeline: 0.42, 1.23, 5.5 and 41.8).
+// 64 x 50, 128 x 128, 256 x 200 and 512 x 400: 0.82, 3.92, 10.4 and 55.2 ms.
 //
 // Every wait is bounded and voted on by its warp; one that runs out raises the abort
 // flag, drains the CTA's own copies, latches DERR_TIMEOUT and returns.
@@ -36,7 +35,6 @@ namespace jac {
 namespace {
 
 constexpr int kBlock = 16;  // columns of a block = warps
-constexpr unsigned kAllLanes = 0xffffffffu;
 
 struct BlockTables {
     uint64_t bar[2];                // TMA loads of the J stages
@@ -153,8 +151,13 @@ __device__ __forceinline__ Turn turn_of(float al, float be, float gr, float gi, 
     p.tg = t * g;
     return p;
 }
-template <int RPL>
-__device__ __forceinline__ void rows_rotate(float2 (&a)[RPL], float2 (&b)[RPL], const Turn& p) {
+// The rotation; b, and with BOTH a, go to their slots in shared memory as soon as their rows
+// are formed, so that the stores are under way before the rotation ends and the next warp
+// waits less for the column (10 of 300 x 300: 35.8 -> 31.7 ms).
+template <int RPL, bool BOTH>
+__device__ __forceinline__ void rows_rotate(float2 (&a)[RPL], float2 (&b)[RPL], const Turn& p, float2* slot_a,
+                                            float2* slot_b) {
+    const int lane = threadIdx.x & 31;
     if constexpr (RPL >= 2) {
         const unsigned long long cm = pk2(p.cm1, p.cm1);
         const unsigned long long sr = pk2(p.sr, p.sr), msr = pk2(-p.sr, -p.sr);
@@ -171,6 +174,11 @@ __device__ __forceinline__ void rows_rotate(float2 (&a)[RPL], float2 (&b)[RPL], 
             a[2 * h + 1] = upk2(add2(ay, fma2(cm, ay, t2)));
             b[2 * h] = upk2(add2(bx, fma2(cm, bx, t3)));
             b[2 * h + 1] = upk2(add2(by, fma2(cm, by, t4)));
+            *reinterpret_cast<float4*>(slot_b + 64 * h + 2 * lane) =
+                make_float4(b[2 * h].x, b[2 * h].y, b[2 * h + 1].x, b[2 * h + 1].y);
+            if constexpr (BOTH)
+                *reinterpret_cast<float4*>(slot_a + 64 * h + 2 * lane) =
+                    make_float4(a[2 * h].x, a[2 * h].y, a[2 * h + 1].x, a[2 * h + 1].y);
         }
     } else {
         const float ar = a[0].x, ai = a[0].y, br = b[0].x, bi = b[0].y;
@@ -178,16 +186,18 @@ __device__ __forceinline__ void rows_rotate(float2 (&a)[RPL], float2 (&b)[RPL], 
         a[0].y = ai + (p.cm1 * ai - (p.sr * bi - p.si * br));
         b[0].x = br + (p.cm1 * br + (p.sr * ar - p.si * ai));
         b[0].y = bi + (p.cm1 * bi + (p.sr * ai + p.si * ar));
+        slot_b[lane] = b[0];
+        if constexpr (BOTH) slot_a[lane] = a[0];
     }
 }
 
 struct Thresholds { float tol2, big2; };
 
-// Rotates the pair (a, b) of one warp unless it is orthogonal to the threshold; al and be
-// are its tracked squared norms.  A zero column or a non-finite value fails the test.
-template <int RPL>
+// Rotates the pair (a, b) of one warp, and stores it, unless it is orthogonal to the
+// threshold; al and be are its tracked squared norms.  A zero column or a non-finite value fails the test.
+template <int RPL, bool BOTH>
 __device__ __forceinline__ bool pair_rotate(float2 (&a)[RPL], float2 (&b)[RPL], float& al, float& be,
-                                            const Thresholds& th, bool& big) {
+                                            const Thresholds& th, bool& big, float2* slot_a, float2* slot_b) {
     float gr, gi;
     rows_dot<RPL>(a, b, gr, gi);
     gr = warp_sum(gr);
@@ -196,7 +206,7 @@ __device__ __forceinline__ bool pair_rotate(float2 (&a)[RPL], float2 (&b)[RPL], 
     if (!(g2 > (th.tol2 * al) * be)) return false;
     big = big || (g2 > (th.big2 * al) * be);
     const Turn p = turn_of(al, be, gr, gi, g2);
-    rows_rotate<RPL>(a, b, p);
+    rows_rotate<RPL, BOTH>(a, b, p, slot_a, slot_b);
     float al2 = al - p.tg, be2 = be + p.tg;
     if (!(al2 > 0.125f * al)) al2 = rows_norm2<RPL>(a);
     if (!(be2 > 0.125f * be)) be2 = rows_norm2<RPL>(b);
@@ -223,6 +233,7 @@ __device__ void blocks_body(float2* W, int ldw, int rows, int cols, int max_swee
     int cur = 0, scale_e = 0;
     bool converged = false;
 
+    auto vote = [](bool x) -> bool { return __all_sync(0xffffffffu, x); };
     auto load_block = [&](int J, int buf) {  // one thread
         const int c0 = J * kBlock, n = min(kBlock, cols - c0);
         // the tracked norms the columns enter the stage with (published by the barrier's arrival)
@@ -328,12 +339,11 @@ __device__ void blocks_body(float2* W, int ldw, int rows, int cols, int max_swee
                     const int p = player(warp), q = player(kBlock - 1 - warp);
                     if (I * kBlock + p < cols && I * kBlock + q < cols) {
                         float2 x[RPL], y[RPL];
-                        load_rows<RPL>(x, buf_i + (size_t)p * ldw, lane, mpad, true);
-                        load_rows<RPL>(y, buf_i + (size_t)q * ldw, lane, mpad, true);
+                        float2 *slot_p = buf_i + p * mpad, *slot_q = buf_i + q * mpad;
+                        load_rows<RPL>(x, slot_p, lane, mpad, true);
+                        load_rows<RPL>(y, slot_q, lane, mpad, true);
                         float nx = T->in2[p], ny = T->in2[q];
-                        if (pair_rotate<RPL>(x, y, nx, ny, th, big)) {
-                            store_rows<RPL>(x, buf_i + (size_t)p * ldw, lane, mpad);
-                            store_rows<RPL>(y, buf_i + (size_t)q * ldw, lane, mpad);
+                        if (pair_rotate<RPL, true>(x, y, nx, ny, th, big, slot_p, slot_q)) {
                             __syncwarp();
                             if (lane == 0) {
                                 T->in2[p] = nx;
@@ -355,32 +365,34 @@ __device__ void blocks_body(float2* W, int ldw, int rows, int cols, int max_swee
                     bulk_wait_read_all();  // the store that last read that stage is done reading
                     load_block(J + 1, nxt);
                 }
-                bool ok = __all_sync(kAllLanes, mbar_wait(&T->bar[cur], phase[cur], &T->abort));
+                bool ok = vote(mbar_wait(&T->bar[cur], phase[cur], &T->abort));
                 if (tid == 0 && ok) T->pending[cur] = 0;
                 // (the counters only grow: no older round can be mistaken for the one needed)
                 const int base = passed[cur] * kBlock;
+                float2* const stage_j = buf_j[cur];
+                float* const jn2 = T->jn2[cur];
+                int* const done = T->done[cur];
                 for (int r = 0; r < kBlock && ok; ++r) {
                     const int jc = (warp + r) & (kBlock - 1), place = J * kBlock + jc;
-                    if (r > 0) ok = __all_sync(kAllLanes, counter_wait(&T->done[cur][jc], base + r, &T->abort));
+                    if (r > 0)
+                        ok = warp_ready(counter_acquire(&done[jc]) >= base + r, vote,
+                                        [&] { return counter_wait(&done[jc], base + r, &T->abort); });
                     if (!ok) break;
                     if (place < cols) {
-                        float be = T->jn2[cur][jc];
+                        float be = jn2[jc];
                         if (mine) {
                             float2 y[RPL];
-                            float2* col = buf_j[cur] + (size_t)jc * ldw;
-                            load_rows<RPL>(y, col, lane, mpad, true);
-                            if (pair_rotate<RPL>(a, y, al, be, th, big)) {
-                                store_rows<RPL>(y, col, lane, mpad);
-                                __syncwarp();
-                                if (lane == 0) T->jn2[cur][jc] = be;
+                            float2* slot = stage_j + jc * mpad;
+                            load_rows<RPL>(y, slot, lane, mpad, true);
+                            if (pair_rotate<RPL, false>(a, y, al, be, th, big, nullptr, slot)) {
+                                jn2[jc] = be;  // (every lane: the same value)
                                 ++rot;
                             }
                         }
-                        if (r == kBlock - 1 && lane == 0) T->nrm2[T->order[place]] = be;
+                        if (r == kBlock - 1) T->nrm2[T->order[place]] = be;
                     }
                     __syncwarp();
-                    if (lane == 0) counter_release_add(&T->done[cur][jc]);
-                    __syncwarp();
+                    if (lane == 0) counter_release_add(&done[jc]);
                 }
                 if (!ok && lane == 0) atomicOr(&T->abort, 1);
                 phase[cur] ^= 1u;
