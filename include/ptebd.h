@@ -215,7 +215,7 @@ int ptebd_set_tensor_cores(ptebd_state* st, int32_t enable);
 
 /* Jacobi block width of the handle's SVDs (no counterpart in the paper: a
  * launch choice).  complex64: 16 (default), the warps and the shared memory of a
- * whole SM for each bond, or 8, at most 4 warps and half the shared memory;
+ * whole SM for each bond, or 8, half of both, so that two bonds share an SM;
  * complex128: always 8.  0 selects the default.  Results are bit-identical run to
  * run at one width (a matrix that only the full shared memory holds takes its
  * first sweeps in twos at width 16, and one by one at width 8).

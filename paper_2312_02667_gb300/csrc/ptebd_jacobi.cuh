@@ -828,10 +828,11 @@ template <typename R> int column_area(int ldw, bool half) {
     const size_t most = (half ? kSmemMax / 2 - 1024 : kSmemMax) - table_bytes<R>();
     return (int)(all < most ? all : most);
 }
-// Compute warps: no more than groups of the widest matrix, at most `most`.
+// Compute warps: no more than groups of the widest matrix, at most `most`; `half`: half of
+// them, so that two CTAs share an SM's registers.
 inline int warps_for(int ldw, bool half, int most) {
-    const int w = ldw / 4 < most ? ldw / 4 : most;
-    return half && w > 4 ? 4 : w;
+    if (half) most /= 2;
+    return ldw / 4 < most ? ldw / 4 : most;
 }
 
 // Where the columns are: streamed from W, in this CTA's shared memory, or spread

@@ -129,8 +129,9 @@ __device__ __forceinline__ void rows_dot(const float2 (&a)[RPL], const float2 (&
 
 // tan (t), cos - 1 and sin e^{i arg g} of the rotation that diagonalises
 // [[al, g], [conj(g), be]], and tan |g|.  t is the smaller root of t^2 + (d / |g|) t - 1 = 0,
-// formed without the quotient; cos is refined by one Newton step, so that
-// cos^2 (1 + t^2) = 1 to rounding with no biased residual.
+// formed without the quotient; cos is refined by one Newton step.  (Taken as a factor, whose
+// rounding leaves the norms 5e-8 to 1.2e-7 too small in the mean; another form would move the
+// results, as another order would.)
 struct Turn { float cm1, sr, si, tg; };
 __device__ __forceinline__ Turn turn_of(float al, float be, float gr, float gi, float g2) {
     const float ig = rsqrtf(g2);
