@@ -25,7 +25,10 @@
  * one workspace buffer on the current device (256-byte aligned, e.g. through
  * the PyTorch caching allocator) and passes them to ptebd_create(); both must
  * stay valid until ptebd_destroy().  The handle itself lives in host memory
- * allocated by ptebd_create and freed by ptebd_destroy.
+ * allocated by ptebd_create and freed by ptebd_destroy, and so does a pinned
+ * buffer of a few KB for the results of small reads (ptebd_get_chi,
+ * ptebd_get_lambda, ptebd_bond_stats, ...); several threads may make such
+ * reads of one state at a time.
  *
  * Streams: every call runs on the stream given at create time (or set later
  * with ptebd_set_stream); calls that return results to the host synchronise

@@ -1363,12 +1363,12 @@ int ptebd_get_chi(ptebd_state* st, int32_t* chi_out) {
 int ptebd_get_lambda(ptebd_state* st, int32_t bond, double* out, int32_t* k) {
     if (!st || !out) return set_err(st, PTEBD_ERR_INVALID, "null argument");
     if (bond < 0 || bond > st->L.n_sites - 2) return set_err(st, PTEBD_ERR_INVALID, "bond out of range");
-    std::vector<double> row(st->L.chip);
+    double row[PTEBD_CHI_LIMIT];
     int32_t kk;
-    const int rc = read_state(st, {{lam_ptr(st, bond), row.size() * sizeof(double), row.data()},
+    const int rc = read_state(st, {{lam_ptr(st, bond), (size_t)st->L.chip * sizeof(double), row},
                                    {at<int32_t>(st->mem, st->L.off_chi) + bond + 1, sizeof kk, &kk}});
     if (rc) return rc;
-    std::memcpy(out, row.data(), (size_t)kk * sizeof(double));
+    std::memcpy(out, row, (size_t)kk * sizeof(double));
     if (k) *k = kk;
     return PTEBD_OK;
 }
