@@ -46,8 +46,8 @@ SM_COUNT = 152
 # the counters no longer describe the kernel.
 JACOBI_SOURCES = ("ptebd_jacobi.cuh", "ptebd_jacobi32.cuh", "ptebd_jacobi.cu")
 JACOBI_TRAFFIC = {
-    # 162.2, 19.2 and 16.2 GB
-    "a86964fc48df961004cb1bf02b82ba254ac80edd455425293faac20f89cb9626": 197.63e9 / 3,
+    # 162.3, 19.2 and 16.2 GB
+    "88c0a710f8102dd0011bb6d9366579f134d4451d4685bcdcb195c10834b2271a": 197.73e9 / 3,
 }
 
 
